@@ -21,7 +21,7 @@
 #include <functional>
 #include <new>
 
-#include "common.cuh"
+#include "loops.cuh"
 
 namespace csl {
 namespace {
@@ -234,15 +234,8 @@ csl_status csl_hatch_layers(const csl_contours* ct, double y0, double spacing, i
         CSL_CUDA(cudaMemsetAsync(small.get(), 0, 16, s));
         if (n_verts > 0 && n_lines > 0) {
             // loop of every vertex, layer of every loop
-            DevBuf vflag((size_t)n_verts * 4, s), loop_of((size_t)n_verts * 4, s);
-            CSL_CUDA(cudaMemsetAsync(vflag.get(), 0, (size_t)n_verts * 4, s));
-            k_mark_i64<<<grid_for(n_loops, 256), 256, 0, s>>>(ct->loop_vert_off, n_loops, n_verts,
-                                                              vflag.as<uint32_t>());
-            CSL_LAUNCH_CHECK("hatch loop starts");
-            exclusive_scan_u32(vflag.as<uint32_t>(), loop_of.as<uint32_t>(), n_verts, nullptr, s);
-            k_incl<<<grid_for(n_verts, 256), 256, 0, s>>>(vflag.as<uint32_t>(),
-                                                          loop_of.as<uint32_t>(), n_verts);
-            CSL_LAUNCH_CHECK("hatch loop of vertex");
+            DevBuf loop_of((size_t)n_verts * 4, s);
+            loops_of_vertices(ct->loop_vert_off, n_loops, n_verts, loop_of.as<uint32_t>(), s);
             DevBuf lflag((size_t)n_loops * 4, s), layer_of((size_t)n_loops * 4, s);
             CSL_CUDA(cudaMemsetAsync(lflag.get(), 0, (size_t)n_loops * 4, s));
             k_mark_i64<<<grid_for(n_layers, 256), 256, 0, s>>>(ct->layer_loop_off, n_layers,

@@ -25,7 +25,7 @@
 
 #include <algorithm>
 
-#include "common.cuh"
+#include "loops.cuh"
 
 namespace csl {
 namespace {
@@ -37,13 +37,6 @@ struct SmConst {
     float m_lo, m_hi;          // mu px and (1 - mu) px
 };
 
-__global__ void k_sm_loop_of(const int64_t* __restrict__ loop_off, int64_t n_loops,
-                             int32_t* __restrict__ vloop) {
-    for (int64_t L = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; L < n_loops;
-         L += (int64_t)gridDim.x * blockDim.x)
-        for (int64_t v = loop_off[L]; v < loop_off[L + 1]; ++v) vloop[v] = (int32_t)L;
-}
-
 __global__ void k_sm_check(const int32_t* __restrict__ eid, int64_t n, int64_t n_ids,
                            uint32_t* bad) {
     bool b = false;
@@ -53,13 +46,13 @@ __global__ void k_sm_check(const int32_t* __restrict__ eid, int64_t n, int64_t n
     if (__syncthreads_or(b) && threadIdx.x == 0) atomicOr(bad, 1u);
 }
 
-__global__ void k_sm_step(const int64_t* __restrict__ loop_off, const int32_t* __restrict__ vloop,
+__global__ void k_sm_step(const int64_t* __restrict__ loop_off, const uint32_t* __restrict__ vloop,
                           const int32_t* __restrict__ eid, const float2* __restrict__ src,
                           int64_t n, SmConst g, float2* __restrict__ dst) {
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n;
          v += (int64_t)gridDim.x * blockDim.x) {
         float2 P = src[v];
-        const int32_t L = vloop[v];
+        const uint32_t L = vloop[v];
         const int64_t a = loop_off[L], b = loop_off[L + 1];
         const int64_t e = eid[v];
         if (b - a >= 3 && e >= 0 && e < g.n_ids) {   // the ids were checked before
@@ -127,12 +120,10 @@ extern "C" csl_status csl_smooth_contours(csl_contours* c, double x0, double y0,
         uint32_t bad = 0;
         read_to_host(&bad, d_bad.get(), 4, s);
         if (bad) fail(CSL_ERR_INVALID_ARG, "edge ids outside the nx x ny grid");
-        k_sm_loop_of<<<grid_for(n_loops, 256), 256, 0, s>>>(c->loop_vert_off, n_loops,
-                                                             d_vloop.as<int32_t>());
-        CSL_LAUNCH_CHECK("smooth vertex loops");
+        loops_of_vertices(c->loop_vert_off, n_loops, n, d_vloop.as<uint32_t>(), s);
         float2* bufs[2] = {reinterpret_cast<float2*>(c->xy), d_tmp.as<float2>()};
         for (int it = 0; it < iterations; ++it) {
-            k_sm_step<<<grid_for(n, 256), 256, 0, s>>>(c->loop_vert_off, d_vloop.as<int32_t>(),
+            k_sm_step<<<grid_for(n, 256), 256, 0, s>>>(c->loop_vert_off, d_vloop.as<uint32_t>(),
                                                        c->edge_id, bufs[it & 1], n, g,
                                                        bufs[(it + 1) & 1]);
             CSL_LAUNCH_CHECK("smooth step");
