@@ -117,3 +117,34 @@ def test_edge_cases_of_the_ray_march():
         lat.render_depth(eye=(0.0, 5.0, 1.0), target=(0.0, 0.0, 1.0), width=3, height=2,
                          step=1e-7)
     assert err.value.code == 1
+
+
+@pytest.mark.parametrize("bundle, far", [(3, False), (40, False), (90, False), (3, True)])
+def test_cell_lists_short_long_and_far_eyes(bundle, far):
+    """Bundles of nearly parallel struts crossing at the origin, so that a cell's
+    list is short, near 64 entries or above them, and an eye from which the
+    samples are looked up one by one; against the oracle."""
+    import paper_2101_05031_gb300 as cs
+    R, rho = 0.5, 0.02 if bundle > 3 else 0.3
+    r = np.random.default_rng(bundle)
+    ends = np.concatenate([r.normal(size=(bundle, 3)) * 0.1 + 2.0 * np.eye(3)[k] for k in range(3)])
+    nodes = np.concatenate([-ends, ends]).astype(np.float32)
+    n = len(ends)
+    edges = np.stack([np.arange(n), np.arange(n) + n], 1).astype(np.int32)
+    radius = np.full(n, rho, np.float32)
+    lat = cs.Lattice(nodes, edges, radius, R=R)
+    cam = dict(eye=(4.1, -5.3, 3.7), target=(0.0, 0.1, 0.0), up=(0.0, 0.0, 1.0), fov_y=0.6,
+               width=19, height=13)
+    if far:
+        cam.update(eye=(4100.0, -5300.0, 3700.0), fov_y=0.0006)
+    step = 0.06
+    depth = lat.render_depth(**cam, step=step, refine=20).cpu().numpy()
+    ref = V.render(nodes, edges, radius, R=R, C=1.0, step=step, refine=20, **cam)
+    # a depth: the float32 rounding of positions, up to 8 ulp of the eye's distance,
+    # over the sine of the incidence (a grazing ray may also decide the other way)
+    tol = 8 * 2.0 ** -24 * np.linalg.norm(cam["eye"]) * 10 + 1e-4
+    hits = sum(np.isfinite(t) for t in ref.values())
+    bad = sum(not (np.isinf(t) and np.isinf(depth[p])) and not abs(depth[p] - t) <= tol
+              for p, t in ref.items())
+    assert hits > 40
+    assert bad <= 0.04 * len(ref), bad
