@@ -43,6 +43,7 @@ struct DmConst {
 struct GridConst {
     double ox, oy, oz, h;
     int32_t nx, ny, nz;
+    double slack;   // of a voxel index estimated from a coordinate, in voxels
 };
 
 // PHYSICAL weight over R^4 (Sec. 3.2): Sigma = w_R4(r) * R^4 I.
@@ -63,38 +64,82 @@ __device__ __forceinline__ float strut_R4I(float px, float py, float pz, float4 
     return segment_term_R4(t0, h2, u.w);
 }
 
-// Mean of sigma((F + W J - C) / T) over the n samples held in shared memory.
-// The same mean by one warp (lane-strided samples, butterfly sum: every lane
-// gets the same value, in a fixed order).
-__device__ __forceinline__ float warp_mean_density(const float* F, const float* J, int n, float W,
-                                                   const DmConst& c) {
+// Mean of sigma((F + W J - C) / T) over the n samples held in shared memory,
+// by one warp (lane-strided samples, butterfly sum: every lane gets the same
+// value, in a fixed order).
+template <bool FAST>
+__device__ __forceinline__ float warp_mean(const float* F, const float* J, int n, float W,
+                                           const DmConst& c) {
     float acc = 0.0f;
     for (int k = threadIdx.x & 31; k < n; k += 32) {
         const float f = F ? F[k] : 0.0f;
         const float x = (f + W * J[k] - c.Cf) * c.inv_T;
-        acc += 1.0f / (1.0f + expf(-x));
+        acc += FAST ? __fdividef(1.0f, 1.0f + __expf(-x)) : 1.0f / (1.0f + expf(-x));
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
     return acc / (float)n;
 }
 
+// warp_mean<false>(...) < target. A bisection step needs only this, so the
+// mean is taken with the approximate exponential and quotient first (9
+// instructions per sample instead of 22): each sample's sigmoid is then off
+// by less than 4e-7 (relative error of __expf (2 + 1.2 |x|) 2^-23, times
+// s (1 - s); 2 ulp of the quotient), and the two sums round by at most
+// (n / 32 + 5) 2^-24 of a mean below 1 each. Within that margin of the target
+// the exact mean decides.
+__device__ __forceinline__ bool warp_mean_below(const float* F, const float* J, int n, float W,
+                                                float target, const DmConst& c) {
+    const float m = warp_mean<true>(F, J, n, W, c);
+    const float margin = 1e-6f + (float)(n / 32 + 8) * 1.3e-7f;
+    if (m + margin < target) return true;
+    if (m - margin >= target) return false;
+    return warp_mean<false>(F, J, n, W, c) < target;
+}
+
+// The ends of the bisection's interval as weights (the same for every
+// tetrahedron and voxel: taken once per kernel).
+struct EndWeights {
+    float lo, hi;
+};
+__device__ __forceinline__ EndWeights end_weights(const DmConst& c) {
+    return EndWeights{weight_R4(c.r0 * 0.5, c), weight_R4(c.r0 * 2.0, c)};
+}
+
 // The ratio s in [1/2, 2] at which the density reaches `target` (the end
 // points when it is out of reach, else `iters` halvings), by one warp;
-// *rho_hi = density at s = 2.
+// *rho_hi = density at s = 2. The weights are FP64 (square root, quotient:
+// about 50 instructions on a pipe that runs at 1/64 of the FP32 rate, so that
+// one weight per halving, the same in all lanes, and exact means throughout
+// took 13.5 ms for 451,000 tetrahedra, now 7.6 ms): every five halvings, lane j takes the weight of node j of the
+// five levels of midpoints below the current interval (node 1 the interval's
+// midpoint, 2 j and 2 j + 1 those of the lower and upper half), and the
+// halvings read theirs from the lanes.
 __device__ float warp_bisect_ratio(const float* F, const float* J, int n, float target,
-                                   const DmConst& c, float* rho_hi) {
-    const float r_hi = warp_mean_density(F, J, n, weight_R4(c.r0 * 2.0, c), c);
+                                   const DmConst& c, const EndWeights& ends, float* rho_hi) {
+    const int lane = threadIdx.x & 31;
+    const float r_hi = warp_mean<false>(F, J, n, ends.hi, c);
     *rho_hi = r_hi;
     if (r_hi <= target) return 2.0f;
-    if (warp_mean_density(F, J, n, weight_R4(c.r0 * 0.5, c), c) >= target) return 0.5f;
+    if (!warp_mean_below(F, J, n, ends.lo, target, c) && target == target) return 0.5f;
     float lo = 0.5f, hi = 2.0f;
-    for (int it = 0; it < c.iters; ++it) {
-        const float mid = 0.5f * (lo + hi);
-        if (warp_mean_density(F, J, n, weight_R4(c.r0 * (double)mid, c), c) < target)
-            lo = mid;
-        else
-            hi = mid;
+    for (int it = 0; it < c.iters; it += 5) {
+        float a = lo, b = hi;
+        for (int level = 30 - __clz(max(lane, 1)); level >= 0; --level) {
+            const float mid = 0.5f * (a + b);
+            if ((lane >> level) & 1) a = mid;
+            else b = mid;
+        }
+        const float w = weight_R4(c.r0 * (double)(0.5f * (a + b)), c);
+        int node = 1;
+        for (int q = it; q < min(it + 5, c.iters); ++q) {
+            const float mid = 0.5f * (lo + hi);
+            const bool below =
+                warp_mean_below(F, J, n, __shfl_sync(0xffffffffu, w, node), target, c);
+            if (below) lo = mid;
+            else hi = mid;
+            node = 2 * node + (below ? 1 : 0);
+        }
     }
     return 0.5f * (lo + hi);
 }
@@ -150,72 +195,112 @@ __device__ double trilinear(const GridConst& g, const float* __restrict__ tgt, d
     return val;
 }
 
-// Voxel index range [lo, hi] along one axis whose centres may lie in [a, b]
-// (one extra voxel on each side; the containment test decides).
+// Voxel index range [lo, hi] along one axis whose centres may lie in [a, b]:
+// slack (in voxels) covers the rounding of the centres and of this estimate,
+// the box and containment tests decide.
 __device__ __forceinline__ void centre_range(double a, double b, double o, double h, int n,
-                                             int& lo, int& hi) {
-    const double fa = fmin(fmax((a - o) / h - 0.5, -2.0), (double)n + 1.0);
-    const double fb = fmin(fmax((b - o) / h - 0.5, -2.0), (double)n + 1.0);
-    lo = max(0, (int)floor(fa) - 1);
-    hi = min(n - 1, (int)ceil(fb) + 1);
+                                             double slack, int& lo, int& hi) {
+    const double fa = fmin(fmax((a - o) / h - 0.5 - slack, -2.0), (double)n + 1.0);
+    const double fb = fmin(fmax((b - o) / h - 0.5 + slack, -2.0), (double)n + 1.0);
+    lo = max(0, (int)ceil(fa));
+    hi = min(n - 1, (int)floor(fb));
 }
 
-// One warp per tetrahedron: the largest target of the contained voxel
-// centres, else the interpolated target at the centroid.
+// One tetrahedron with its box and the voxels whose centres may lie in it.
+struct TetBox {
+    double3 v[4];
+    double D, lo[3], hi[3];
+    int i0, j0, k0, ni, nj, nk;
+    int64_t cnt;
+
+    __device__ __forceinline__ void load(const float4* __restrict__ tv, const GridConst& g) {
+        for (int k = 0; k < 4; ++k) {
+            const float4 q = tv[k];
+            v[k] = make_double3(q.x, q.y, q.z);
+        }
+        D = orient(v[0], v[1], v[2], v[3]);
+        lo[0] = fmin(fmin(v[0].x, v[1].x), fmin(v[2].x, v[3].x));
+        hi[0] = fmax(fmax(v[0].x, v[1].x), fmax(v[2].x, v[3].x));
+        lo[1] = fmin(fmin(v[0].y, v[1].y), fmin(v[2].y, v[3].y));
+        hi[1] = fmax(fmax(v[0].y, v[1].y), fmax(v[2].y, v[3].y));
+        lo[2] = fmin(fmin(v[0].z, v[1].z), fmin(v[2].z, v[3].z));
+        hi[2] = fmax(fmax(v[0].z, v[1].z), fmax(v[2].z, v[3].z));
+        int i1, j1, k1;
+        centre_range(lo[0], hi[0], g.ox, g.h, g.nx, g.slack, i0, i1);
+        centre_range(lo[1], hi[1], g.oy, g.h, g.ny, g.slack, j0, j1);
+        centre_range(lo[2], hi[2], g.oz, g.h, g.nz, g.slack, k0, k1);
+        ni = i1 - i0 + 1;
+        nj = j1 - j0 + 1;
+        nk = k1 - k0 + 1;
+        cnt = (D != 0.0 && ni > 0 && nj > 0 && nk > 0) ? (int64_t)ni * nj * nk : 0;
+    }
+    // the target of voxel (i, j, k) where the tetrahedron contains its centre
+    __device__ __forceinline__ void take(int i, int j, int k, const GridConst& g,
+                                         const float* __restrict__ tgt, double& best,
+                                         bool& found) const {
+        const double3 p = make_double3(g.ox + g.h * ((double)i + 0.5),
+                                       g.oy + g.h * ((double)j + 0.5),
+                                       g.oz + g.h * ((double)k + 0.5));
+        // a centre outside the bounding box cannot be contained
+        const bool in_box = p.x >= lo[0] && p.x <= hi[0] && p.y >= lo[1] && p.y <= hi[1] &&
+                            p.z >= lo[2] && p.z <= hi[2];
+        if (in_box && contains(v, D, p)) {
+            found = true;
+            best = fmax(best, (double)tgt[((int64_t)k * g.ny + j) * g.nx + i]);
+        }
+    }
+};
+
+// The largest target of the voxel centres that a tetrahedron contains, else the
+// interpolated target at the centroid. A lane per tetrahedron while it has
+// few candidate centres (FP64 set-up that is the same in every lane of a warp
+// costs as much for one tetrahedron as for 32: with a warp per tetrahedron 451,000
+// of them took 6.7 ms, now 0.29 ms); the warp shares the candidates of the
+// others.
+constexpr int kDmOwn = 16;
 __global__ void k_dm_target(const float4* __restrict__ tv, int64_t n_tets, GridConst g,
                             const float* __restrict__ tgt, double* __restrict__ out) {
     const int lane = threadIdx.x & 31;
-    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-    for (int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; t < n_tets;
-         t += warps) {
-        double3 v[4];
-        for (int k = 0; k < 4; ++k) {
-            const float4 q = tv[4 * t + k];
-            v[k] = make_double3(q.x, q.y, q.z);
-        }
-        const double D = orient(v[0], v[1], v[2], v[3]);
-        const double xmin = fmin(fmin(v[0].x, v[1].x), fmin(v[2].x, v[3].x));
-        const double xmax = fmax(fmax(v[0].x, v[1].x), fmax(v[2].x, v[3].x));
-        const double ymin = fmin(fmin(v[0].y, v[1].y), fmin(v[2].y, v[3].y));
-        const double ymax = fmax(fmax(v[0].y, v[1].y), fmax(v[2].y, v[3].y));
-        const double zmin = fmin(fmin(v[0].z, v[1].z), fmin(v[2].z, v[3].z));
-        const double zmax = fmax(fmax(v[0].z, v[1].z), fmax(v[2].z, v[3].z));
-        int i0, i1, j0, j1, k0, k1;
-        centre_range(xmin, xmax, g.ox, g.h, g.nx, i0, i1);
-        centre_range(ymin, ymax, g.oy, g.h, g.ny, j0, j1);
-        centre_range(zmin, zmax, g.oz, g.h, g.nz, k0, k1);
-        const int64_t ni = i1 - i0 + 1, nj = j1 - j0 + 1, nk = k1 - k0 + 1;
-        const int64_t cnt = (D != 0.0 && ni > 0 && nj > 0 && nk > 0) ? ni * nj * nk : 0;
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t t0 = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31u); t0 < n_tets;
+         t0 += stride) {
+        const int64_t t = t0 + lane;
         double best = -INFINITY;
         bool found = false;
-        for (int64_t q = lane; q < cnt; q += 32) {
-            const int i = i0 + (int)(q % ni);
-            const int j = j0 + (int)((q / ni) % nj);
-            const int k = k0 + (int)(q / (ni * nj));
-            const double3 p = make_double3(g.ox + g.h * ((double)i + 0.5),
-                                           g.oy + g.h * ((double)j + 0.5),
-                                           g.oz + g.h * ((double)k + 0.5));
-            // a centre outside the bounding box cannot be contained
-            const bool in_box = p.x >= xmin && p.x <= xmax && p.y >= ymin && p.y <= ymax &&
-                                p.z >= zmin && p.z <= zmax;
-            if (in_box && contains(v, D, p)) {
-                found = true;
-                best = fmax(best, (double)tgt[((int64_t)k * g.ny + j) * g.nx + i]);
-            }
+        int64_t cnt = 0;
+        double3 c = make_double3(0.0, 0.0, 0.0);
+        if (t < n_tets) {
+            TetBox b;
+            b.load(tv + 4 * t, g);
+            c = make_double3((b.v[0].x + b.v[1].x + b.v[2].x + b.v[3].x) * 0.25,
+                             (b.v[0].y + b.v[1].y + b.v[2].y + b.v[3].y) * 0.25,
+                             (b.v[0].z + b.v[1].z + b.v[2].z + b.v[3].z) * 0.25);
+            cnt = b.cnt;
+            if (cnt <= kDmOwn)
+                for (int q = 0; q < (int)cnt; ++q)
+                    b.take(b.i0 + q % b.ni, b.j0 + q / b.ni % b.nj, b.k0 + q / (b.ni * b.nj), g,
+                           tgt, best, found);
         }
+        uint32_t many = __ballot_sync(0xffffffffu, cnt > kDmOwn);
+        while (many) {
+            const int src = __ffs(many) - 1;
+            many &= many - 1u;
+            TetBox b;
+            b.load(tv + 4 * (t0 + src), g);
+            double m = -INFINITY;
+            bool f = false;
+            for (int64_t q = lane; q < b.cnt; q += 32)
+                b.take(b.i0 + (int)(q % b.ni), b.j0 + (int)(q / b.ni % b.nj),
+                       b.k0 + (int)(q / ((int64_t)b.ni * b.nj)), g, tgt, m, f);
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) best = fmax(best, __shfl_xor_sync(0xffffffffu, best, o));
-        found = __any_sync(0xffffffffu, found);
-        if (lane == 0) {
-            if (found) {
-                out[t] = best;
-            } else {
-                const double3 c = make_double3((v[0].x + v[1].x + v[2].x + v[3].x) * 0.25,
-                                               (v[0].y + v[1].y + v[2].y + v[3].y) * 0.25,
-                                               (v[0].z + v[1].z + v[2].z + v[3].z) * 0.25);
-                out[t] = trilinear(g, tgt, c);
+            for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+            f = __any_sync(0xffffffffu, f);
+            if (lane == src) {
+                best = m;
+                found = f;
             }
         }
+        if (t < n_tets) out[t] = found ? best : trilinear(g, tgt, c);
     }
 }
 
@@ -232,6 +317,7 @@ k_dm_tet(const float4* __restrict__ tv, const double* __restrict__ target, int64
     extern __shared__ float s_dyn[];
     const int lane = threadIdx.x & 31;
     float* s_J = s_dyn + (size_t)(threadIdx.x >> 5) * n_samples;
+    const EndWeights ends = end_weights(c);
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
     for (int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; t < n_tets;
          t += warps) {
@@ -268,7 +354,7 @@ k_dm_tet(const float4* __restrict__ tv, const double* __restrict__ target, int64
         }
         __syncwarp();
         float r_hi;
-        const float s = warp_bisect_ratio(nullptr, s_J, n_samples, (float)target[t], c, &r_hi);
+        const float s = warp_bisect_ratio(nullptr, s_J, n_samples, (float)target[t], c, ends, &r_hi);
         if (lane == 0) {
             rho_star[t] = r_hi;
             ratio[t] = s;
@@ -407,6 +493,7 @@ k_dm_voxel(const uint32_t* __restrict__ vals, const uint32_t* __restrict__ vbeg,
     const int n = m * m * m;
     const int64_t n_vox = (int64_t)g.nx * g.ny * g.nz;
     const float hf = (float)g.h, inv_m = 1.0f / (float)m;
+    const EndWeights ends = end_weights(c);
     for (int64_t v = blockIdx.x; v < n_vox; v += gridDim.x) {
         const uint32_t b0 = vbeg[v], b1 = vend[v];
         if (b0 >= b1) {
@@ -464,7 +551,7 @@ k_dm_voxel(const uint32_t* __restrict__ vals, const uint32_t* __restrict__ vbeg,
         }
         if (threadIdx.x < 32) {   // one warp bisects; no block barrier per step
             float r_hi;
-            const float s = warp_bisect_ratio(s_F, s_J, n, tgt[v], c, &r_hi);
+            const float s = warp_bisect_ratio(s_F, s_J, n, tgt[v], c, ends, &r_hi);
             if (threadIdx.x == 0) vox_ratio[v] = s;
         }
         __syncthreads();   // s_F, s_J are rewritten by the next voxel
@@ -601,6 +688,9 @@ extern "C" csl_status csl_density_match(const float* nodes, int64_t n_nodes, con
         g.nx = vox->dims[0];
         g.ny = vox->dims[1];
         g.nz = vox->dims[2];
+        g.slack = 0.0;
+        for (int k = 0; k < 3; ++k)
+            g.slack = std::max(g.slack, 1e-3 + 1e-15 * (fabs(vox->origin[k]) / g.h + vox->dims[k]));
         const int n_samples = p->tet_n * p->tet_n * p->tet_n;
         // warps per block of the tetrahedron kernel: their J slices fit 48 KB
         const int tet_warps = std::max(1, std::min(kDmThreads / 32, 12288 / n_samples));
@@ -643,7 +733,7 @@ extern "C" csl_status csl_density_match(const float* nodes, int64_t n_nodes, con
             double* tgt_d = d_target.as<double>() + t0;
             float* rho_d = d_rho.as<float>() + t0;
             float* rat_d = d_ratio.as<float>() + t0;
-            k_dm_target<<<grid_for(nc * 32, 256), 256, 0, s>>>(d_tv.as<float4>(), nc, g,
+            k_dm_target<<<grid_for(nc, 128), 128, 0, s>>>(d_tv.as<float4>(), nc, g,
                                                                d_tgt.as<float>(), tgt_d);
             CSL_LAUNCH_CHECK("density targets");
             k_dm_tet<<<grid_for(nc * 32, tet_threads), tet_threads, tet_smem, s>>>(

@@ -213,3 +213,19 @@ def test_full_workload_sampled_against_the_oracle():
     rad = got["radius"].astype(np.float64)
     assert np.all(rad >= 0.5 * r0 * (1 - 1e-6))
     assert np.all(rad <= r0 * got["step3_ratio"].astype(np.float64) * (1 + 1e-6))
+
+
+@pytest.mark.parametrize("voxel, cubes", [(0.9, 2), (1.7, 3), (4.0, 5), (30.0, 3)])
+def test_targets_over_candidate_counts(voxel, cubes):
+    """Step 1's targets where a tetrahedron holds hundreds of voxel centres, about
+    as many as a lane takes alone, few and none (the interpolated ones)."""
+    import paper_2101_05031_gb300 as cs
+    nodes, tets = synth.kuhn_tet_mesh((cubes,) * 3, 4.0, 0.1, seed=31)
+    grid = synth.graded_target_grid((0.0,) * 3, (4.0 * cubes,) * 3, voxel, period=9.0)
+    r = np.random.default_rng(7)
+    grid["target"] = (grid["target"] * r.uniform(0.5, 1.0, grid["target"].shape)).astype(np.float32)
+    got = cs.density_match(nodes, tets, grid, r_min=0.1, tet_n=2, vox_m=2, max_depth=0, iters=7)
+    assert np.array_equal(got["tets"], tets)
+    want = np.array([D.tet_target(grid, nodes[t].astype(np.float64)) for t in tets])
+    # 8 products and sums in FP64: below 1e-14 relative; a contained centre's is exact
+    assert np.allclose(got["target"], want, rtol=1e-13, atol=0.0)
