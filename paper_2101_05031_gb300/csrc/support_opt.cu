@@ -16,6 +16,7 @@
 // initial volume, and J decreases. Rounds repeat until nothing moves. All
 // arithmetic is FP64 in one fixed order (the build compiles device code with
 // --fmad=false).
+#include <limits.h>
 #include <math.h>
 
 #include <algorithm>
@@ -29,12 +30,17 @@ namespace csl {
 namespace {
 
 constexpr int kPoThreads = 128;
+// k_po_move: one warp per block, so that the warps of a colour spread evenly
+// over the SMs (864 warps of the FP64 pipe's work on 152 SMs: 42 us of the
+// busiest SM's pipe with 6 warps, 57 us with two blocks of 4)
+constexpr int kPoMoveThreads = 32;
 
 struct PoConst {
     double tx, ty, tz, alpha;
     double a[6];
     double step, ball, min_volume;
     int32_t backtracks;
+    float g2_max;   // bound of |g''| on [0, pi / 2], for the FP32 screening
 };
 
 // g(theta) of Eq. 12 and its derivative, by Horner (0, 0 for theta <= alpha).
@@ -48,21 +54,46 @@ __device__ __forceinline__ void g_dg(double th, const PoConst& c, double& g, dou
     }
 }
 
-// One warp evaluates J(v) at (vx, vy, vz) over the vertex's edges [b, e) of
-// the CSR: each lane computes the terms of its edges, then the sums are taken
-// in edge order (lane by lane through shuffles), the order of the sequential
-// definition. With grad != nullptr also the gradient. Every lane returns the
-// same values.
-__device__ double warp_J(double vx, double vy, double vz, const int32_t* __restrict__ nbr,
-                         const double* __restrict__ rad, int64_t b, int64_t e,
-                         const double* __restrict__ pos, const PoConst& c, double* grad) {
-    const int lane = threadIdx.x & 31;
-    double N = 0.0, D = 0.0;
-    double dN[3] = {0.0, 0.0, 0.0}, dD[3] = {0.0, 0.0, 0.0};
+// The G lanes (16 or 32) of a warp that work on one vertex.
+template <int G>
+struct Group {
+    int lane;        // in the group
+    unsigned mask;   // its lanes in the warp
+    __device__ __forceinline__ Group() {
+        const int l = threadIdx.x & 31;
+        lane = l & (G - 1);
+        mask = (G == 32 ? 0xffffffffu : 0xffffu) << (l & ~(G - 1));
+    }
+    __device__ __forceinline__ bool any(bool p) const { return (__ballot_sync(mask, p) & mask) != 0; }
+    template <class T>
+    __device__ __forceinline__ T from(T v, int src) const {
+        return __shfl_sync(mask, v, src, G);
+    }
+    __device__ __forceinline__ float sum(float v) const {
+#pragma unroll
+        for (int o = G / 2; o > 0; o >>= 1) v += __shfl_xor_sync(mask, v, o, G);
+        return v;
+    }
+};
+
+// A group evaluates J(v) at (vx, vy, vz) over the vertex's edges [b, e) of the
+// CSR: each lane computes the terms of its edges; then lane k takes component
+// k of the sums (N, D and, with GRAD, the gradients of N and D) through shared
+// memory, in edge order, the order of the sequential definition: one FP64
+// addition per edge for all components together (the pipe takes 32 lanes as
+// long as one). Every lane returns the same values. sm: G * (GRAD ? 8 : 2)
+// doubles of the group's own.
+template <int G, bool GRAD>
+__device__ double group_J(const Group<G>& gr, double vx, double vy, double vz,
+                          const int32_t* __restrict__ nbr, const double* __restrict__ rad,
+                          int64_t b, int64_t e, const double* __restrict__ pos, const PoConst& c,
+                          double* sm, double* grad) {
+    constexpr int K = GRAD ? 8 : 2;
     const double tk[3] = {c.tx, c.ty, c.tz};
-    for (int64_t base = b; base < e; base += 32) {
-        const int64_t i = base + lane;
-        double tN = 0.0, tD = 0.0, tdN[3] = {0.0, 0.0, 0.0}, tdD[3] = {0.0, 0.0, 0.0};
+    double acc = 0.0;
+    for (int64_t base = b; base < e; base += G) {
+        const int64_t i = base + gr.lane;
+        double t[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};   // N, D, dN, dD
         bool live = false;
         if (i < e) {
             const int32_t w = nbr[i];
@@ -77,51 +108,42 @@ __device__ double warp_J(double vx, double vy, double vz, const int32_t* __restr
                 const double th = acos(cs);
                 double g, dg;
                 g_dg(th, c, g, dg);
-                const double dL[3] = {d[0] / L, d[1] / L, d[2] / L};
-                tN = r * L * g;
-                tD = r * L;
-                if (grad) {
-                    for (int k = 0; k < 3; ++k) tdD[k] = r * dL[k];
+                t[0] = r * L * g;
+                t[1] = r * L;
+                if (GRAD) {
+                    const double dL[3] = {d[0] / L, d[1] / L, d[2] / L};
+                    for (int k = 0; k < 3; ++k) t[5 + k] = r * dL[k];
                     if (g != 0.0 || dg != 0.0) {
                         const double sg = copysign(1.0, s);
                         const double s2 = sqrt(fmax(1.0 - cs * cs, 1e-300));
                         for (int k = 0; k < 3; ++k) {
                             const double dc = (sg * tk[k] - cs * dL[k]) / L;
                             const double dth = -dc / s2;
-                            tdN[k] = r * (dL[k] * g + L * dg * dth);
+                            t[2 + k] = r * (dL[k] * g + L * dg * dth);
                         }
                     }
                 }
             }
         }
-        const int n = (int)min((int64_t)32, e - base);
-        const unsigned live_mask = __ballot_sync(0xffffffffu, live);
-        for (int j = 0; j < n; ++j) {   // edge order
-            const double xN = __shfl_sync(0xffffffffu, tN, j);
-            const double xD = __shfl_sync(0xffffffffu, tD, j);
-            double xdN[3], xdD[3];
-            if (grad)
-                for (int k = 0; k < 3; ++k) {
-                    xdN[k] = __shfl_sync(0xffffffffu, tdN[k], j);
-                    xdD[k] = __shfl_sync(0xffffffffu, tdD[k], j);
-                }
-            if (!((live_mask >> j) & 1u)) continue;   // a zero-length edge adds nothing
-            N += xN;
-            D += xD;
-            if (grad)
-                for (int k = 0; k < 3; ++k) {
-                    dD[k] += xdD[k];
-                    dN[k] += xdN[k];
-                }
+        const int n = (int)min((int64_t)G, e - base);
+        const unsigned live_mask =
+            __ballot_sync(gr.mask, live) >> (G == 32 ? 0 : (threadIdx.x & 16));
+#pragma unroll
+        for (int k = 0; k < K; ++k) sm[k * G + gr.lane] = t[k];
+        __syncwarp(gr.mask);
+        if (gr.lane < K)
+            for (int j = 0; j < n; ++j)   // edge order; a zero-length edge adds nothing
+                if ((live_mask >> j) & 1u) acc += sm[gr.lane * G + j];
+        __syncwarp(gr.mask);
+    }
+    const double N = gr.from(acc, 0), D = gr.from(acc, 1);
+    if (GRAD) {
+        for (int k = 0; k < 3; ++k) {
+            const double dN = gr.from(acc, 2 + k), dD = gr.from(acc, 5 + k);
+            grad[k] = D == 0.0 ? 0.0 : (dN * D - N * dD) / (D * D);
         }
     }
-    if (D == 0.0) {
-        if (grad) grad[0] = grad[1] = grad[2] = 0.0;
-        return 0.0;
-    }
-    if (grad)
-        for (int k = 0; k < 3; ++k) grad[k] = (dN[k] * D - N * dD[k]) / (D * D);
-    return N / D;
+    return D == 0.0 ? 0.0 : N / D;
 }
 
 __device__ __forceinline__ double orient(const double* a, const double* b, const double* c,
@@ -177,9 +199,114 @@ __global__ void k_po_vol0(const int4* __restrict__ tets, int64_t n, const double
     }
 }
 
-// One colour: a warp per vertex of the list (no two share an edge). The
-// lanes share the edge terms and the incident tetrahedra's checks; the trials
-// of the backtracking run in order.
+// A trial's tests in FP32, on offsets from the vertex's position p0 taken in
+// FP64 and rounded once (relative error 2^-24; the step's offset 2^-23).
+// Each returns +1 / -1 where the FP64 test must come out true / false whatever
+// the rounding of this evaluation, 0 where it might not: then the FP64 test
+// decides. FP64 runs at 1/64 of the FP32 rate here, and most trials are far
+// from every bound.
+struct Screen {
+    // this lane's edge: offset p0 - neighbour and radius (r = 0: none)
+    float ex, ey, ez, r;
+    // this lane's tetrahedra (up to 2): the three other corners' offsets from
+    // p0, the sign that turns their determinant into the oriented volume times
+    // sign(vol0), and |vol0| min_volume
+    float q[2][9], sign[2], least[2];
+    int n_tets;
+};
+
+// |cand - o| <= rb?
+__device__ __forceinline__ int screen_ball(const float (&w)[3], const float (&dl)[3], float rb) {
+    const float x = w[0] + dl[0], y = w[1] + dl[1], z = w[2] + dl[2];
+    const float dist = sqrtf(x * x + y * y + z * z);
+    const float size = fabsf(w[0]) + fabsf(w[1]) + fabsf(w[2]) + fabsf(dl[0]) + fabsf(dl[1]) +
+                       fabsf(dl[2]);
+    if (!(size > 1e-15f && size < 1e15f)) return 0;   // squares in range
+    const float m = 1e-6f * (size + rb);
+    return dist + m < rb ? 1 : (dist - m > rb ? -1 : 0);
+}
+
+// Does tetrahedron k keep its orientation and its least volume? A product of
+// three offsets errs by less than 3e-6 of the product of their sizes.
+__device__ __forceinline__ int screen_volume(const Screen& S, int k, const float (&dl)[3]) {
+    float e[9], size = 1.0f;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        float a = 0.0f;
+#pragma unroll
+        for (int x = 0; x < 3; ++x) {
+            e[3 * i + x] = S.q[k][3 * i + x] - dl[x];
+            a += fabsf(S.q[k][3 * i + x]) + fabsf(dl[x]);
+        }
+        size *= a;
+    }
+    const float det = e[0] * (e[4] * e[8] - e[5] * e[7]) - e[1] * (e[3] * e[8] - e[5] * e[6]) +
+                      e[2] * (e[3] * e[7] - e[4] * e[6]);
+    if (!(size > 1e-30f && size < 1e30f)) return 0;
+    const float y = S.sign[k] * det, m = 3e-6f * size;
+    return y - m > S.least[k] * (1.0f + 1e-6f) ? 1
+                                                : (y + m < S.least[k] * (1.0f - 1e-6f) ? -1 : 0);
+}
+
+// J(cand) < J0? The angle's error follows from the offset's (acos moves by at
+// most 1.5 e / sin near its argument, g by |g'| e + g'' e^2); an angle within
+// its error of alpha, or an error above 1e-4, leaves the question open.
+template <int G>
+__device__ __forceinline__ int screen_J(const Group<G>& gr, const Screen& S, const float (&dl)[3],
+                                        float J0, const PoConst& c) {
+    float N = 0.0f, D = 0.0f, eN = 0.0f, eD = 0.0f;
+    bool open = false;
+    if (S.r > 0.0f) {
+        const float x = S.ex + dl[0], y = S.ey + dl[1], z = S.ez + dl[2];
+        const float L2 = x * x + y * y + z * z;
+        const float L = sqrtf(L2);
+        const float size = fabsf(S.ex) + fabsf(S.ey) + fabsf(S.ez) + fabsf(dl[0]) + fabsf(dl[1]) +
+                           fabsf(dl[2]);
+        const float ed = __fdividef(4e-7f * size, L);
+        const float cs = fminf(
+            __fdividef(fabsf(x * (float)c.tx + y * (float)c.ty + z * (float)c.tz), L), 1.0f);
+        const float sin2 = fmaxf(1.0f - cs * cs, 0.0f);
+        const float ecs = 2.0f * ed + 6e-7f;
+        const float eth = (ecs < 0.25f * sin2 ? 1.5f * ecs * rsqrtf(sin2) : 1.6f * sqrtf(ecs)) +
+                          1e-6f;
+        const float th = acosf(cs), over = th - (float)c.alpha;
+        const float rL = S.r * L;
+        open = !(L2 > 1e-30f && L2 < 1e30f && rL > 1e-30f && rL < 1e30f && eth <= 1e-4f &&
+                 fabsf(over) > eth);
+        float g = 0.0f, dg = 0.0f, eg = 0.0f;
+        if (over > 0.0f) {
+            float size_g = 0.0f;   // sum |a_i| th^i: Horner rounds by less than 11 2^-24 of it
+#pragma unroll
+            for (int i = 5; i >= 0; --i) {
+                dg = dg * th + g;
+                g = g * th + (float)c.a[i];
+                size_g = size_g * th + fabsf((float)c.a[i]);
+            }
+            eg = eth * (fabsf(dg) + eth * c.g2_max) + 1.5e-6f * size_g;
+        }
+        N = rL * g;
+        D = rL;
+        eN = rL * eg + fabsf(N) * (ed + 6e-6f);
+        eD = rL * (ed + 6e-6f);
+    }
+    open = gr.any(open);
+    N = gr.sum(N);
+    D = gr.sum(D);
+    eN = gr.sum(eN);
+    eD = gr.sum(eD);
+    if (open || !(eD < 0.1f * D)) return 0;
+    const float J = N / D;
+    const float m = 2.0f * (eN + fabsf(J) * eD) / D + 1e-6f * (fabsf(J) + fabsf(J0));
+    return J + m < J0 ? 1 : (J - m > J0 ? -1 : 0);
+}
+
+// One colour: G lanes per vertex of the list (no two share an edge). The lanes
+// share the edge terms and the incident tetrahedra's checks; the trials of the
+// backtracking run in order. Bound by the FP64 pipe and its latency: the
+// gradient and J at the vertex's position are FP64 (two vertices per warp where
+// degrees allow), the trials' tests are screened in FP32 (of 373,000 values of
+// J in a call on 93,750 tetrahedra 21,000 stay open). That call's 136 launches:
+// 17.0 ms with a warp per vertex in FP64 throughout, 7.5 ms now.
 //
 // A vertex's move depends only on its own position and its neighbours' (all
 // the vertices of its tetrahedra) besides constants; so a vertex that did not
@@ -187,7 +314,8 @@ __global__ void k_po_vol0(const int4* __restrict__ tets, int64_t n, const double
 // moved since (moved_at of it and of its neighbours older than that step)
 // would not move now either, and is skipped: the result of the sequential
 // sweep exactly, without re-evaluating the calm part of the mesh.
-__global__ void __launch_bounds__(kPoThreads)
+template <int G>
+__global__ void __launch_bounds__(kPoMoveThreads)
 k_po_move(const int32_t* __restrict__ list, int64_t n, double* __restrict__ pos,
           const double* __restrict__ o, const double* __restrict__ tau0,
           const int64_t* __restrict__ e_off, const int32_t* __restrict__ nbr,
@@ -195,51 +323,124 @@ k_po_move(const int32_t* __restrict__ list, int64_t n, double* __restrict__ pos,
           const int32_t* __restrict__ vt, const int4* __restrict__ tets,
           const double* __restrict__ vol0, PoConst c, int32_t step,
           int32_t* __restrict__ moved_at, int32_t* __restrict__ calm_at, unsigned int* moves) {
-    const int lane = threadIdx.x & 31;
-    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-    for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < n; i += warps) {
+    __shared__ double s_terms[kPoMoveThreads / G][8 * G];
+    const Group<G> gr;
+    double* sm = s_terms[threadIdx.x / G];
+    const int64_t groups = (int64_t)gridDim.x * (kPoMoveThreads / G);
+    for (int64_t i = ((int64_t)blockIdx.x * kPoMoveThreads + threadIdx.x) / G; i < n; i += groups) {
         const int32_t v = list[i];
         const int64_t eb = e_off[v], ee = e_off[v + 1];
         const int32_t ca = calm_at[v];
         if (ca >= 0 && moved_at[v] < ca) {   // calm before: has the star moved since?
             bool moved = false;
-            for (int64_t q = eb + lane; q < ee; q += 32) moved |= moved_at[nbr[q]] > ca;
-            if (!__any_sync(0xffffffffu, moved)) continue;
+            for (int64_t q = eb + gr.lane; q < ee; q += G) moved |= moved_at[nbr[q]] > ca;
+            if (!gr.any(moved)) continue;
         }
         double* pv = pos + 3 * (int64_t)v;
         const double p0 = pv[0], p1 = pv[1], p2 = pv[2];
         double grad[3];
-        const double J0 = warp_J(p0, p1, p2, nbr, rad, eb, ee, pos, c, grad);
+        const double J0 = group_J<G, true>(gr, p0, p1, p2, nbr, rad, eb, ee, pos, c, sm, grad);
         const double gn = sqrt(grad[0] * grad[0] + grad[1] * grad[1] + grad[2] * grad[2]);
-        bool went = false;
         if (gn == 0.0) {
-            if (lane == 0) calm_at[v] = step;
+            if (gr.lane == 0) calm_at[v] = step;
             continue;
         }
         const double u[3] = {grad[0] / gn, grad[1] / gn, grad[2] / gn};
         const double* ov = o + 3 * (int64_t)v;
         const double rb = c.ball * tau0[v];
         const int64_t tb = vt_off[v], te = vt_off[v + 1];
-        double s = c.step * tau0[v];
-        for (int it = 0; it <= c.backtracks; ++it, s *= 0.5) {
-            const double cand[3] = {p0 - s * u[0], p1 - s * u[1], p2 - s * u[2]};
-            const double dx = cand[0] - ov[0], dy = cand[1] - ov[1], dz = cand[2] - ov[2];
-            if (sqrt(dx * dx + dy * dy + dz * dz) > rb) continue;
-            bool ok = true;
-            for (int64_t q = tb + lane; q < te; q += 32) {
+        // the screening's data: an edge and up to two tetrahedra per lane
+        const bool screened = ee - eb <= G && te - tb <= 2 * G;
+        Screen S;
+        S.r = 0.0f;
+        S.n_tets = 0;
+        if (screened) {
+            if (eb + gr.lane < ee) {
+                const double* pw = pos + 3 * (int64_t)nbr[eb + gr.lane];
+                S.ex = (float)(p0 - pw[0]);
+                S.ey = (float)(p1 - pw[1]);
+                S.ez = (float)(p2 - pw[2]);
+                S.r = (float)rad[eb + gr.lane];
+            }
+#pragma unroll
+            for (int m = 0; m < 2; ++m) {
+                const int64_t q = tb + gr.lane + m * G;
+                if (q >= te) continue;
+                S.n_tets = m + 1;
                 const int32_t ti = vt[q] >> 2, k = vt[q] & 3;
                 const int4 t = tets[ti];
                 const int32_t id[4] = {t.x, t.y, t.z, t.w};
-                const double* P[4];
-                for (int j = 0; j < 4; ++j) P[j] = j == k ? cand : pos + 3 * (int64_t)id[j];
-                const double vol = orient(P[0], P[1], P[2], P[3]);
-                ok = ok && vol * vol0[ti] > 0.0 && fabs(vol) >= c.min_volume * fabs(vol0[ti]);
+#pragma unroll
+                for (int j = 0; j < 3; ++j) {
+                    const double* pw = pos + 3 * (int64_t)id[kFace[k][j]];
+                    S.q[m][3 * j] = (float)(pw[0] - p0);
+                    S.q[m][3 * j + 1] = (float)(pw[1] - p1);
+                    S.q[m][3 * j + 2] = (float)(pw[2] - p2);
+                }
+                // moving corner k to the front is an odd permutation for odd k
+                const double v0 = vol0[ti];
+                S.sign[m] = v0 == 0.0 ? NAN : (((k & 1) != 0) != (v0 < 0.0) ? -1.0f : 1.0f);
+                S.least[m] = (float)(c.min_volume * fabs(v0));
             }
-            if (!__all_sync(0xffffffffu, ok)) continue;
-            const double J1 = warp_J(cand[0], cand[1], cand[2], nbr, rad, eb, ee, pos, c, nullptr);
-            if (J1 < J0) {
-                __syncwarp();   // every lane has read pv before lane 0 writes it
-                if (lane == 0) {
+        }
+        const float w[3] = {(float)(p0 - ov[0]), (float)(p1 - ov[1]), (float)(p2 - ov[2])};
+        const float uf[3] = {(float)u[0], (float)u[1], (float)u[2]};
+        bool went = false;
+        const double s0 = c.step * tau0[v];
+        float sf = (float)s0;
+        for (int it = 0; it <= c.backtracks; ++it, sf *= 0.5f) {
+            const float dl[3] = {-sf * uf[0], -sf * uf[1], -sf * uf[2]};
+            // the FP64 candidate, where it is needed: s0 halved `it` times (exact)
+            auto candidate = [&](double (&cand)[3]) {
+                const double s = s0 * __hiloint2double((1023 - it) << 20, 0);
+                cand[0] = p0 - s * u[0];
+                cand[1] = p1 - s * u[1];
+                cand[2] = p2 - s * u[2];
+            };
+            double cand[3];
+            int in = screened ? screen_ball(w, dl, (float)rb) : 0;
+            if (in == 0) {
+                candidate(cand);
+                const double dx = cand[0] - ov[0], dy = cand[1] - ov[1], dz = cand[2] - ov[2];
+                in = sqrt(dx * dx + dy * dy + dz * dz) > rb ? -1 : 1;
+            }
+            if (in < 0) continue;
+            int vol[2] = {1, 1};
+            bool bad = false, open = !screened;
+            if (screened) {
+#pragma unroll
+                for (int m = 0; m < 2; ++m)
+                    if (m < S.n_tets) vol[m] = screen_volume(S, m, dl);
+                bad = gr.any(vol[0] < 0 || vol[1] < 0);
+                open = gr.any(vol[0] == 0 || vol[1] == 0);
+            }
+            if (bad) continue;
+            if (open) {
+                candidate(cand);
+                bool ok = true;
+                for (int64_t q = tb + gr.lane, m = 0; q < te; q += G, ++m) {
+                    if (screened && vol[m] > 0) continue;
+                    const int32_t ti = vt[q] >> 2, k = vt[q] & 3;
+                    const int4 t = tets[ti];
+                    const int32_t id[4] = {t.x, t.y, t.z, t.w};
+                    const double* P[4];
+                    for (int j = 0; j < 4; ++j) P[j] = j == k ? cand : pos + 3 * (int64_t)id[j];
+                    const double vc = orient(P[0], P[1], P[2], P[3]);
+                    ok = ok && vc * vol0[ti] > 0.0 && fabs(vc) >= c.min_volume * fabs(vol0[ti]);
+                }
+                if (gr.any(!ok)) continue;
+            }
+            int less = screened ? screen_J(gr, S, dl, (float)J0, c) : 0;
+            if (less == 0) {
+                candidate(cand);
+                const double J1 = group_J<G, false>(gr, cand[0], cand[1], cand[2], nbr, rad, eb, ee,
+                                                    pos, c, sm, nullptr);
+                less = J1 < J0 ? 1 : -1;
+            }
+            if (less > 0) {
+                __syncwarp(gr.mask);   // every lane has read pv before lane 0 writes it
+                if (gr.lane == 0) {
+                    candidate(cand);
                     pv[0] = cand[0];
                     pv[1] = cand[1];
                     pv[2] = cand[2];
@@ -250,7 +451,7 @@ k_po_move(const int32_t* __restrict__ list, int64_t n, double* __restrict__ pos,
                 break;
             }
         }
-        if (!went && lane == 0) calm_at[v] = step;
+        if (!went && gr.lane == 0) calm_at[v] = step;
     }
 }
 
@@ -363,6 +564,9 @@ extern "C" csl_status csl_support_optimize(float* nodes, int64_t n_nodes, const 
         c.ball = p->ball;
         c.min_volume = p->min_volume;
         c.backtracks = p->backtracks;
+        double g2_max = 0.0;
+        for (int i = 2; i < 6; ++i) g2_max += i * (i - 1) * fabs(p->a[i]) * pow(1.6, i - 2);
+        c.g2_max = (float)g2_max;
         cudaStream_t s = (cudaStream_t)stream;
 
         // vertex -> (tetrahedron, corner)
@@ -526,6 +730,13 @@ extern "C" csl_status csl_support_optimize(float* nodes, int64_t n_nodes, const 
                 d_tets.as<int4>(), n_tets, d_pos.as<double>(), d_vol0.as<double>());
             CSL_LAUNCH_CHECK("initial volumes");
         }
+        // two vertices per warp where every vertex's edges fit 16 lanes and its
+        // tetrahedra two per lane (the interior of a Kuhn mesh: 14 and 24)
+        bool half_warps = true;
+        for (int64_t i = 0; i < n_list && half_warps; ++i) {
+            const int32_t v = list[i];
+            half_warps = e_off[v + 1] - e_off[v] <= 16 && vt_off[v + 1] - vt_off[v] <= 32;
+        }
         csl_po_result r = {};
         r.n_colours = n_col;
         metrics(d_edges, d_er, n_e, d_pos, c, d_part, d_tot, s, &r.gamma_before, &r.psi_before);
@@ -534,7 +745,8 @@ extern "C" csl_status csl_support_optimize(float* nodes, int64_t n_nodes, const 
             for (int32_t k = 0; k < n_col; ++k) {
                 const int64_t b = col_off[k], n = col_off[k + 1] - b;
                 if (!n) continue;
-                k_po_move<<<grid_for(n * 32, kPoThreads), kPoThreads, 0, s>>>(
+                auto move = half_warps ? k_po_move<16> : k_po_move<32>;
+                move<<<grid_for(n * (half_warps ? 16 : 32), kPoMoveThreads, INT_MAX), kPoMoveThreads, 0, s>>>(
                     d_list.as<int32_t>() + b, n, d_pos.as<double>(), d_o.as<double>(),
                     d_tau.as<double>(), d_eoff.as<int64_t>(), d_nbr.as<int32_t>(),
                     d_rad.as<double>(), d_vtoff.as<int64_t>(), d_vt.as<int32_t>(),

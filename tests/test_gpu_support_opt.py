@@ -93,3 +93,43 @@ def test_full_workload_first_round_sampled():
     v0, v1 = _volumes(x0, t), _volumes(x1, t)
     assert np.all(v0 * v1 > 0.0)
     assert np.all(np.abs(v1) >= st.min_volume * np.abs(v0) * (1 - 1e-3))
+
+
+def _fan_mesh(n_rim, seed):
+    """Two hubs above each other inside a rim of n_rim nodes and two poles: hubs of
+    n_rim + 2 edges and 3 n_rim or so tetrahedra (more than a lane group screens)."""
+    r = np.random.default_rng(seed)
+    a = 2 * np.pi * np.arange(n_rim) / n_rim
+    rim = np.stack([np.cos(a), np.sin(a), 0.2 * r.uniform(-1, 1, n_rim)], 1)
+    nodes = np.concatenate([[[0.05, 0.0, 0.3], [-0.04, 0.03, -0.35], [0, 0, 2.0], [0, 0, -2.0]], rim])
+    tets = []
+    for k in range(n_rim):
+        i, j = 4 + k, 4 + (k + 1) % n_rim
+        tets += [[0, i, j, 2], [1, j, i, 3], [0, j, i, 1]]
+    return nodes.astype(np.float32), np.array(tets, np.int32)
+
+
+@pytest.mark.parametrize("case", ["fan14", "fan30", "fan70", "kuhn_tiny", "kuhn_huge", "alpha_small",
+                                  "alpha_0", "volume_strict", "volume_free", "steep_g"])
+def test_screened_trials_decide_as_fp64(case):
+    """Where a trial's tests are taken in FP32 first: degrees below, at and above the
+    lanes of a vertex, scales at which FP32 products would leave its range, angles
+    near alpha and near 0, tight and no volume limits, large coefficients."""
+    kw = dict(max_rounds=12)
+    if case.startswith("fan"):
+        nodes, tets = _fan_mesh(int(case[3:]), 3)
+    else:
+        nodes, tets = synth.kuhn_tet_mesh((3, 3, 3), 1.0, 0.18, seed=synth.SEED_BASE + 12)
+    scale = {"kuhn_tiny": 1e-13, "kuhn_huge": 1e12}.get(case, 1.0)
+    nodes = (nodes.astype(np.float64) * scale).astype(np.float32)
+    kw.update({"alpha_small": dict(alpha=0.05), "alpha_0": dict(alpha=0.0),
+               "volume_strict": dict(min_volume=0.85), "volume_free": dict(min_volume=0.0)}
+              .get(case, {}))
+    import paper_2101_05031_gb300 as cs
+    a = (3e5, -7e5, 2e5, 4e5, -3e5, 1e5) if case == "steep_g" else P.PAPER_A
+    ref = P.optimize(nodes, tets, None, a=a, **kw)
+    got = cs.support_optimize(nodes, tets, None, coeffs=a, **kw)
+    assert got["moves_per_round"] == ref["moves"]
+    x = ref["nodes"]
+    assert np.all(np.abs(got["nodes"].astype(np.float64) - x) <= 1e-6 * (np.abs(x) + scale))
+    assert sum(ref["moves"]) > 0
