@@ -29,6 +29,7 @@
 // branch-free.
 #include <math.h>
 
+#include <algorithm>
 #include <vector>
 
 #include "field_tile.cuh"
@@ -64,7 +65,11 @@ struct FieldConst {
 // with one arrival), phase: its parity, kept by the caller across tiles.
 // Returns false (after setting ST_TIMEOUT in *c.err) when a copy never
 // completed; the caller must then stop using the barrier.
-template <int S, bool COUNT>
+//
+// PX: pixel rows per thread (1, or 2: a warp then owns 8 x 8 pixels and the CTA
+// has 4 warps; rows j and j + 4 of a thread share x, so dx and dz, the walk
+// over the records and the layer tests).
+template <int S, int PX, bool COUNT>
 __device__ __forceinline__ bool field_tile(const csl_rec* __restrict__ recs,
                                            const uint32_t* __restrict__ tstart,
                                            const uint32_t* __restrict__ tend, const FieldConst& c,
@@ -79,13 +84,16 @@ __device__ __forceinline__ bool field_tile(const csl_rec* __restrict__ recs,
     const uint32_t beg = tstart[key], end = tend[key];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int wx = warp & 1, wy = warp >> 1;
-    const int il = wx * 8 + (lane & 7), jl = wy * 4 + (lane >> 3);
+    constexpr int kThreads = kFieldThreads / PX;
+    const int il = wx * 8 + (lane & 7), jl = wy * 4 * PX + (lane >> 3);
     const int l0 = slab * S;
     const int nl = min(S, c.n_layers - l0);
 
-    float acc[S];
+    float acc[S][PX];
 #pragma unroll
-    for (int l = 0; l < S; ++l) acc[l] = 0.0f;
+    for (int l = 0; l < S; ++l)
+#pragma unroll
+        for (int k = 0; k < PX; ++k) acc[l][k] = 0.0f;
     uint32_t n_nonzero = 0, n_eval = 0;
 
     if (end > beg) {
@@ -93,7 +101,9 @@ __device__ __forceinline__ bool field_tile(const csl_rec* __restrict__ recs,
         const float2 ox = c.org_x[tx], oy = c.org_y[ty], oz = c.org_z[slab];
         const float oxh = ox.x, oxl = ox.y, oyh = oy.x, oyl = oy.y, ozh = oz.x, ozl = oz.y;
         const float pxl = ((float)il + 0.5f) * c.fpx;
-        const float pyl = ((float)jl + 0.5f) * c.fpx;
+        float pyl[PX];
+#pragma unroll
+        for (int k = 0; k < PX; ++k) pyl[k] = ((float)(jl + 4 * k) + 0.5f) * c.fpx;
         const TileCull cull = c.tc;
 
         for (uint32_t c0 = beg; c0 < end; c0 += kFieldThreads) {
@@ -110,50 +120,70 @@ __device__ __forceinline__ bool field_tile(const csl_rec* __restrict__ recs,
                 return false;
             }
             phase ^= 1u;
-            if ((int)threadIdx.x < cnt) {
-                const float4 r0 = s_rec[threadIdx.x][0], r1 = s_rec[threadIdx.x][1];
-                s_rec[threadIdx.x][0] =
+#pragma unroll 1
+            for (int r = threadIdx.x; r < cnt; r += kThreads) {
+                const float4 r0 = s_rec[r][0], r1 = s_rec[r][1];
+                s_rec[r][0] =
                     make_float4((r0.x - oxh) - oxl, (r0.y - oyh) - oyl, (r0.z - ozh) - ozl, r0.w);
-                s_rec[threadIdx.x][1] = make_float4(r1.x, r1.y, r1.z, r1.w * cull.inv_R4);
-                s_mask[threadIdx.x] = 0;
+                s_rec[r][1] = make_float4(r1.x, r1.y, r1.z, r1.w * cull.inv_R4);
+                s_mask[r] = 0;
             }
             __syncthreads();
             // cull masks: one (record, layer) item per thread; byte l of s_mask[r]
             // holds the warps of layer l
-            for (int item = threadIdx.x; item < cnt * nl; item += kFieldThreads) {
-                const int r = item % cnt, l = item / cnt;
-                reinterpret_cast<uint8_t*>(s_mask)[8 * r + l] =
-                    (uint8_t)cull_layer(s_rec[r][0], s_rec[r][1], l, cull);
+#pragma unroll 1
+            for (int item = threadIdx.x; item < cnt * S; item += kThreads) {
+                const int r = item / S, l = item % S;
+                if (l < nl)
+                    reinterpret_cast<uint8_t*>(s_mask)[8 * r + l] =
+                        (uint8_t)cull_layer<PX>(s_rec[r][0], s_rec[r][1], l, cull);
             }
             __syncthreads();
+#pragma unroll 1
             for (int i0 = 0; i0 < cnt; i0 += 32) {
                 const int i = i0 + lane;
                 const uint32_t wm = i < cnt ? warp_layers(s_mask[i], warp) : 0u;
                 uint32_t ball = __ballot_sync(0xffffffffu, wm != 0u);
+#pragma unroll 1
                 while (ball) {
                     const int b = __ffs(ball) - 1;
                     ball &= ball - 1u;
                     const uint32_t lm = __shfl_sync(0xffffffffu, wm, b);
                     const float4 A = s_rec[i0 + b][0], B = s_rec[i0 + b][1];
-                    const float dx = pxl - A.x, dy = pyl - A.y;
-                    const float txy = fmaf(dy, B.x, dx * A.w);
+                    const float dx = pxl - A.x;
+                    float dy[PX], txy[PX];
+#pragma unroll
+                    for (int k = 0; k < PX; ++k) {
+                        dy[k] = pyl[k] - A.y;
+                        txy[k] = fmaf(dy[k], B.x, dx * A.w);
+                    }
 #pragma unroll
                     for (int l = 0; l < S; ++l) {
                         if (lm & (1u << l)) {
                             const float dz = (float)l * c.fdz - A.z;
-                            const float t0 = fmaf(dz, B.y, txy);
-                            const float ex = fmaf(-t0, A.w, dx);
-                            const float ey = fmaf(-t0, B.x, dy);
-                            const float ez = fmaf(-t0, B.y, dz);
-                            const float d2 = fmaf(ez, ez, fmaf(ey, ey, ex * ex));
-                            const float h2 = fmaxf(c.R2 - d2, 0.0f);
-                            // the rest only when some pixel of the warp is within R
-                            if (__any_sync(0xffffffffu, h2 > 0.0f)) {
-                                const float I = segment_term_R4(t0, h2, B.z);
-                                acc[l] = fmaf(B.w, I, acc[l]);
-                                if (COUNT) {
-                                    n_nonzero += I > 0.0f;
-                                    ++n_eval;
+                            float t0[PX], h2[PX];
+                            bool near = PX == 2;
+#pragma unroll
+                            for (int k = 0; k < PX; ++k) {
+                                t0[k] = fmaf(dz, B.y, txy[k]);
+                                const float ex = fmaf(-t0[k], A.w, dx);
+                                const float ey = fmaf(-t0[k], B.x, dy[k]);
+                                const float ez = fmaf(-t0[k], B.y, dz);
+                                const float d2 = fmaf(ez, ez, fmaf(ey, ey, ex * ex));
+                                h2[k] = fmaxf(c.R2 - d2, 0.0f);
+                                near |= h2[k] > 0.0f;
+                            }
+                            // the rest only when some pixel of the warp is within R (with
+                            // two rows per thread, for wide supports, nearly always)
+                            if (PX == 2 || __any_sync(0xffffffffu, near)) {
+#pragma unroll
+                                for (int k = 0; k < PX; ++k) {
+                                    const float I = segment_term_R4(t0[k], h2[k], B.z);
+                                    acc[l][k] = fmaf(B.w, I, acc[l][k]);
+                                    if (COUNT) {
+                                        n_nonzero += I > 0.0f;
+                                        ++n_eval;
+                                    }
                                 }
                             }
                         }
@@ -176,30 +206,34 @@ __device__ __forceinline__ bool field_tile(const csl_rec* __restrict__ recs,
         if (lane == 0 && t) atomicAdd(n_pairs, t);
         if (lane == 0 && e) atomicAdd(n_pairs + 1, e);
     }
-    const int gi = tx * kTile + il, gj = ty * kTile + jl;
-    const bool in_grid = gi < c.nx && gj < c.ny;
-    if (in_grid && sigma) {   // no Sigma plane when only the mask is wanted
+    const int gi = tx * kTile + il;
 #pragma unroll
-        for (int l = 0; l < S; ++l)
-            if (l < nl) sigma[((int64_t)(l0 + l) * c.ny + gj) * c.nx + gi] = acc[l];
-    }
-    if (mask) {
-        // inside bits of the warp's 8 x 4 block: one byte per pixel row, OR-ed
-        // into the padded row (pixel i is padded sample i + 1)
-        const int I0 = tx * kTile + wx * 8 + 1;
-        const int sh = I0 & 31;
+    for (int k = 0; k < PX; ++k) {
+        const int gj = ty * kTile + jl + 4 * k;
+        const bool in_grid = gi < c.nx && gj < c.ny;
+        if (in_grid && sigma) {   // no Sigma plane when only the mask is wanted
 #pragma unroll
-        for (int l = 0; l < S; ++l) {
-            if (l >= nl) break;
-            const uint32_t ball = __ballot_sync(0xffffffffu, in_grid && acc[l] >= c.C);
-            if (lane < 4) {
-                const uint32_t byte = (ball >> (8 * lane)) & 0xffu;
-                if (byte) {
-                    const int J = ty * kTile + wy * 4 + lane + 1;
-                    uint32_t* row = mask + (int64_t)(l0 + l) * c.mask_wpl + (int64_t)J * c.mwr;
-                    atomicOr(row + (I0 >> 5), byte << sh);
-                    const uint32_t hi = sh > 24 ? byte >> (32 - sh) : 0u;
-                    if (hi) atomicOr(row + (I0 >> 5) + 1, hi);
+            for (int l = 0; l < S; ++l)
+                if (l < nl) sigma[((int64_t)(l0 + l) * c.ny + gj) * c.nx + gi] = acc[l][k];
+        }
+        if (mask) {
+            // inside bits of 8 x 4 pixels: one byte per pixel row, OR-ed into the
+            // padded row (pixel i is padded sample i + 1)
+            const int I0 = tx * kTile + wx * 8 + 1;
+            const int sh = I0 & 31;
+#pragma unroll
+            for (int l = 0; l < S; ++l) {
+                if (l >= nl) break;
+                const uint32_t ball = __ballot_sync(0xffffffffu, in_grid && acc[l][k] >= c.C);
+                if (lane < 4) {
+                    const uint32_t byte = (ball >> (8 * lane)) & 0xffu;
+                    if (byte) {
+                        const int J = ty * kTile + wy * 4 * PX + 4 * k + lane + 1;
+                        uint32_t* row = mask + (int64_t)(l0 + l) * c.mask_wpl + (int64_t)J * c.mwr;
+                        atomicOr(row + (I0 >> 5), byte << sh);
+                        const uint32_t hi = sh > 24 ? byte >> (32 - sh) : 0u;
+                        if (hi) atomicOr(row + (I0 >> 5) + 1, hi);
+                    }
                 }
             }
         }
@@ -207,8 +241,8 @@ __device__ __forceinline__ bool field_tile(const csl_rec* __restrict__ recs,
     return true;
 }
 
-template <int S, bool COUNT>
-__global__ void __launch_bounds__(kFieldThreads, 8)
+template <int S, int PX, bool COUNT>
+__global__ void __launch_bounds__(kFieldThreads / PX, PX == 2 ? 10 : 8)
 k_field(const csl_rec* __restrict__ recs, const uint32_t* __restrict__ tstart,
         const uint32_t* __restrict__ tend, FieldConst c, float* __restrict__ sigma,
         uint32_t* __restrict__ mask, unsigned long long* __restrict__ n_pairs) {
@@ -219,7 +253,7 @@ k_field(const csl_rec* __restrict__ recs, const uint32_t* __restrict__ tstart,
     }
     __syncthreads();
     uint32_t phase = 0;
-    field_tile<S, COUNT>(recs, tstart, tend, c, sigma, mask, n_pairs, blockIdx.x, blockIdx.y,
+    field_tile<S, PX, COUNT>(recs, tstart, tend, c, sigma, mask, n_pairs, blockIdx.x, blockIdx.y,
                          &bar, phase);
 }
 
@@ -237,8 +271,8 @@ static_assert(sizeof(FieldJob) % 4 == 0, "FieldJob is copied as 32-bit words");
 // Persistent field kernel over the (job, slab, tile) items of a batch: each
 // CTA takes the next item from a shared counter, in the order `order` gives
 // (longest tile lists first, so the short ones fill the tail).
-template <int S>
-__global__ void __launch_bounds__(kFieldThreads, 6)
+template <int S, int PX>
+__global__ void __launch_bounds__(kFieldThreads / PX, 6)
 k_field_batch(const FieldJob* __restrict__ jobs, const uint2* __restrict__ items,
               const uint32_t* __restrict__ order, uint32_t n_items, uint32_t* counter) {
     __shared__ uint32_t s_item;
@@ -260,12 +294,12 @@ k_field_batch(const FieldJob* __restrict__ jobs, const uint2* __restrict__ items
         if (item.x != cur_job) {   // consecutive items often belong to the same job
             cur_job = item.x;
             const uint32_t* src = reinterpret_cast<const uint32_t*>(jobs + item.x);
-            for (int i = threadIdx.x; i < (int)(sizeof(FieldJob) / 4); i += kFieldThreads)
+            for (int i = threadIdx.x; i < (int)(sizeof(FieldJob) / 4); i += kFieldThreads / PX)
                 reinterpret_cast<uint32_t*>(&s_job)[i] = src[i];
             __syncthreads();
         }
         const uint32_t n_tiles = (uint32_t)s_job.c.n_tiles;
-        if (!field_tile<S, false>(s_job.recs, s_job.tstart, s_job.tend, s_job.c, s_job.sigma,
+        if (!field_tile<S, PX, false>(s_job.recs, s_job.tstart, s_job.tend, s_job.c, s_job.sigma,
                                   s_job.mask, nullptr, (int)(item.y % n_tiles),
                                   (int)(item.y / n_tiles), &bar, phase))
             break;   // a bulk copy gave up (reported): this CTA takes no more items
@@ -334,7 +368,7 @@ namespace {
 
 // Kernel constants of a chunk; org = the chunk's origin tables (ntx + nty +
 // n_slabs float2, as k_origins writes them).
-FieldConst make_field_const(const ChunkGeom& g, float C, const float2* org) {
+FieldConst make_field_const(const ChunkGeom& g, float C, const float2* org, int rows) {
     FieldConst c;
     c.C = C;
     c.org_x = org;
@@ -359,8 +393,10 @@ FieldConst make_field_const(const ChunkGeom& g, float C, const float2* org) {
     c.fdz = (float)g.dz;
     c.cull = (float)(g.R * (1.0 + 1e-5) + 1e-6);
     {
-        // pixel centres of a warp's 8 x 4 block lie within 3.5 x 1.5 pixels of its centre
-        double hd = g.px * sqrt(3.5 * 3.5 + 1.5 * 1.5) * (1.0 + 1e-5);
+        // pixel centres of a warp's block of 8 x 4 rows pixels lie within 3.5 x
+        // (2 rows - 1/2) pixels of its centre
+        const double hy = 2.0 * rows - 0.5;
+        double hd = g.px * sqrt(3.5 * 3.5 + hy * hy) * (1.0 + 1e-5);
         double r = (double)c.cull + hd;
         c.cull_line2 = (float)(r * r);
     }
@@ -371,6 +407,16 @@ FieldConst make_field_const(const ChunkGeom& g, float C, const float2* org) {
     c.tc.inv_R4 = c.inv_R4;
     return c;
 }
+
+// Pixel rows per thread of the block kernel. Two halve the visits of records and
+// their layer tests, and cost lanes where a support covers few pixels (1,332
+// against 1,151 million evaluated terms for 818 million nonzero ones at R = 26
+// px, with 17 % fewer instructions in all). Field of 2000^2 px x 200 layers at R
+// = 26 px: 20.4 ms with one row, 17.5 with two (90 % issue); at 15 px (12 batched
+// lattices) 8.0 and 6.8 ms, at 10.5 px (780^2 x 190) 4.11 and 3.91 ms. Below, one
+// row: there the automatic choice takes the footprint kernel, and the volume
+// fraction's samples (R = 5 px) keep 8 x 4 blocks.
+int rows_per_thread(const ChunkGeom& g) { return g.R >= 10.0 * g.px ? 2 : 1; }
 
 void launch_origins(const ChunkGeom& g, float2* org, cudaStream_t s) {
     k_origins<<<(unsigned)ceil_div(g.ntx + g.nty + g.n_slabs, 128), 128, 0, s>>>(
@@ -393,20 +439,22 @@ void field_chunk(const csl_lattice* L, const ChunkGeom& g, const SlabBins& bins,
     }
     if (g.fused || fv) fail(CSL_ERR_INVALID_ARG, "the fused pass needs the footprint kernel");
     if (g.T != kTile) fail(CSL_ERR_INVALID_ARG, "the block field kernel takes 16-pixel tiles");
-    FieldConst c = make_field_const(g, C, org_d.as<float2>());
+    const int rows = rows_per_thread(g);
+    FieldConst c = make_field_const(g, C, org_d.as<float2>(), rows);
     c.err = L->status.as<uint32_t>();
     dim3 grid((unsigned)c.n_tiles, (unsigned)g.n_slabs);
     const csl_rec* recs = bins.recs.as<csl_rec>();
     const uint32_t* ts = bins.tile_start.as<uint32_t>();
     const uint32_t* te = bins.tile_end.as<uint32_t>();
+#define CSL_FIELD_LAUNCH(SV, PXV, CNT)                                                       \
+    k_field<SV, PXV, CNT><<<grid, kFieldThreads / PXV, 0, s>>>(recs, ts, te, c, sigma, mask,  \
+                                                               count_pairs)
 #define CSL_FIELD_CASE(SV)                                                                    \
     case SV:                                                                                  \
-        if (count_pairs)                                                                      \
-            k_field<SV, true><<<grid, kFieldThreads, 0, s>>>(recs, ts, te, c, sigma, mask,    \
-                                                             count_pairs);                    \
-        else                                                                                  \
-            k_field<SV, false><<<grid, kFieldThreads, 0, s>>>(recs, ts, te, c, sigma, mask,   \
-                                                              nullptr);                       \
+        if (rows == 2 && count_pairs) CSL_FIELD_LAUNCH(SV, 2, true);                          \
+        else if (rows == 2) CSL_FIELD_LAUNCH(SV, 2, false);                                   \
+        else if (count_pairs) CSL_FIELD_LAUNCH(SV, 1, true);                                  \
+        else CSL_FIELD_LAUNCH(SV, 1, false);                                                  \
         break;
     switch (g.S) {
         CSL_FIELD_CASE(1)
@@ -416,6 +464,7 @@ void field_chunk(const csl_lattice* L, const ChunkGeom& g, const SlabBins& bins,
         default: fail(CSL_ERR_INVALID_ARG, "slab depth must be 1, 2, 4 or 8");
     }
 #undef CSL_FIELD_CASE
+#undef CSL_FIELD_LAUNCH
     CSL_LAUNCH_CHECK("field");
 }
 
@@ -442,6 +491,8 @@ void field_batch_prepare(const std::vector<FieldBatchJob>& jobs, FieldBatch& fb,
     fb.T = T;
     fb.K = K;
     fb.n_items = off[n_jobs];
+    fb.rows = 2;   // one kernel for all jobs
+    for (const FieldBatchJob& J : jobs) fb.rows = std::min(fb.rows, rows_per_thread(J.g));
     fb.origins.alloc_persistent(n_org * sizeof(float2));
     std::vector<FieldJob> hj(n_jobs);
     std::vector<const float2*> orgs(n_jobs);
@@ -452,7 +503,7 @@ void field_batch_prepare(const std::vector<FieldBatchJob>& jobs, FieldBatch& fb,
         orgs[j] = org;
         launch_origins(J.g, org, s);
         o += (size_t)J.g.ntx + J.g.nty + J.g.n_slabs;
-        hj[j].c = make_field_const(J.g, (float)J.L->C, org);
+        hj[j].c = make_field_const(J.g, (float)J.L->C, org, fb.rows);
         hj[j].c.err = J.err;
         hj[j].recs = J.bins->recs.as<csl_rec>();
         hj[j].tstart = J.bins->tile_start.as<uint32_t>();
@@ -504,13 +555,24 @@ void field_batch_run(FieldBatch& fb, int n_ctas, cudaStream_t s) {
         fp_batch_launch(fb.fp_jobs.get(), items, order, n, counter, fb.T, fb.S, fb.K, n_ctas, s);
         return;
     }
+    // with two pixel rows per thread a CTA has half the threads: twice as many CTAs
+#define CSL_FIELD_CASE(SV)                                                                     \
+    case SV:                                                                                   \
+        if (fb.rows == 2)                                                                      \
+            k_field_batch<SV, 2><<<2 * n_ctas, kFieldThreads / 2, 0, s>>>(jobs, items, order,  \
+                                                                          n, counter);         \
+        else                                                                                   \
+            k_field_batch<SV, 1><<<n_ctas, kFieldThreads, 0, s>>>(jobs, items, order, n,       \
+                                                                  counter);                    \
+        break;
     switch (fb.S) {
-        case 1: k_field_batch<1><<<n_ctas, kFieldThreads, 0, s>>>(jobs, items, order, n, counter); break;
-        case 2: k_field_batch<2><<<n_ctas, kFieldThreads, 0, s>>>(jobs, items, order, n, counter); break;
-        case 4: k_field_batch<4><<<n_ctas, kFieldThreads, 0, s>>>(jobs, items, order, n, counter); break;
-        case 8: k_field_batch<8><<<n_ctas, kFieldThreads, 0, s>>>(jobs, items, order, n, counter); break;
+        CSL_FIELD_CASE(1)
+        CSL_FIELD_CASE(2)
+        CSL_FIELD_CASE(4)
+        CSL_FIELD_CASE(8)
         default: fail(CSL_ERR_INVALID_ARG, "slab depth must be 1, 2, 4 or 8");
     }
+#undef CSL_FIELD_CASE
     CSL_LAUNCH_CHECK("batch field");
 }
 

@@ -204,14 +204,17 @@ __device__ __forceinline__ bool row_span(const float4 A, const float4 B, float z
     return i0 <= i1;
 }
 
-// The warps of one layer l whose 8 x 4 block the staged edge (A, B) may reach
-// (the test of stage_record for a single layer): bit w set for warp w.
+// The warps of one layer l whose block of 8 x 4 PX pixels the staged edge (A, B)
+// may reach (the test of stage_record for a single layer; c.cull_line2 for that
+// block): bit w set for warp w of the tile's 8 / PX.
+template <int PX>
 __device__ __forceinline__ uint32_t cull_layer(const float4 A, const float4 B, int l,
                                                const TileCull& c) {
     const float ax = A.x, ay = A.y, az = A.z, ux = A.w, uy = B.x, uz = B.y, len = B.z;
     const float zl = (float)l * c.fdz;
     float t_lo = 0.0f, t_hi = len;
     if (uz > 1e-12f) {
+        // approximate: these bounds move by far less than cull's slack
         const float inv_uz = 1.0f / uz;
         t_lo = fmaxf((zl - c.cull - az) * inv_uz, 0.0f);
         t_hi = fminf((zl + c.cull - az) * inv_uz, len);
@@ -226,11 +229,11 @@ __device__ __forceinline__ uint32_t cull_layer(const float4 A, const float4 B, i
     const float qz = zl - az;
     uint32_t m = 0;
 #pragma unroll
-    for (int w = 0; w < kTileWarps; ++w) {
+    for (int w = 0; w < kTileWarps / PX; ++w) {
         const float rx0 = ((float)((w & 1) * 8) + 0.5f) * c.fpx;
         const float rx1 = ((float)((w & 1) * 8) + 7.5f) * c.fpx;
-        const float ry0 = ((float)((w >> 1) * 4) + 0.5f) * c.fpx;
-        const float ry1 = ((float)((w >> 1) * 4) + 3.5f) * c.fpx;
+        const float ry0 = ((float)((w >> 1) * 4 * PX) + 0.5f) * c.fpx;
+        const float ry1 = ((float)((w >> 1) * 4 * PX) + (4 * PX - 0.5f)) * c.fpx;
         if (xmax >= rx0 && xmin <= rx1 && ymax >= ry0 && ymin <= ry1) {
             const float qx = 0.5f * (rx0 + rx1) - ax;
             const float qy = 0.5f * (ry0 + ry1) - ay;

@@ -121,6 +121,7 @@ struct FieldBatch {
     int64_t n_items = 0;
     int S = 0;
     int kernel = kFieldBlock, T = kTile, K = 256;   // the jobs' field kernel, tile, staging chunk
+    int rows = 1;   // block kernel: pixel rows per thread
 };
 // One-time tables (synchronises s).
 void field_batch_prepare(const std::vector<FieldBatchJob>& jobs, FieldBatch& fb, cudaStream_t s);
