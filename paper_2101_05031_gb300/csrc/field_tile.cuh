@@ -1,6 +1,6 @@
-// Device helpers shared by the field kernel and the volume-fraction adjoint:
-// staging one edge record for a (16x16-pixel tile, slab) CTA, the per-warp
-// cull mask, and the closed-form segment integral (Eq. 7) by 3-point
+// Device helpers shared by the field kernels, the volume-fraction adjoint and the
+// ray caster: bulk copies, one edge record in a tile's frame, the per-warp cull
+// mask of the block kernel, and the closed-form segment integral (Eq. 7) by 3-point
 // Gauss-Legendre on the clipped interval.
 #pragma once
 
@@ -70,65 +70,9 @@ __device__ __forceinline__ float sqrt_approx(float x) {
     return r;
 }
 
-// Loads record rp, converts it to coordinates relative to the tile corner and
-// the slab's first layer plane (each given as a (hi, lo) float pair) and
-// returns its cull mask: bit w * 8 + l is set when the edge's support (radius
-// cull) may reach a pixel centre of warp w's 8 x 4 block at layer l < nl,
-// i.e. when the block meets the xy box of the edge clipped to |z - z_l| <= cull
-// grown by cull, and the block's centre lies within cull + half-diagonal of
-// the edge's line. A = (ax, ay, az, ux), B = (uy, uz, len, w / R^4).
-__device__ __forceinline__ uint64_t stage_record(const csl_rec* rp_rec, float oxh, float oxl,
-                                                 float oyh, float oyl, float ozh, float ozl, int nl,
-                                                 const TileCull& c, float4& A, float4& B) {
-    const float4* rp = reinterpret_cast<const float4*>(rp_rec);
-    const float4 r0 = __ldg(rp), r1 = __ldg(rp + 1);
-    const float ax = (r0.x - oxh) - oxl;
-    const float ay = (r0.y - oyh) - oyl;
-    const float az = (r0.z - ozh) - ozl;
-    const float ux = r0.w, uy = r1.x, uz = r1.y, len = r1.z;
-    A = make_float4(ax, ay, az, ux);
-    B = make_float4(uy, uz, len, r1.w * c.inv_R4);
-    uint64_t m = 0;
-    const float inv_uz = uz > 1e-12f ? 1.0f / uz : 0.0f;
-#pragma unroll 1
-    for (int l = 0; l < nl; ++l) {
-        const float zl = (float)l * c.fdz;
-        float t_lo = 0.0f, t_hi = len;
-        if (uz > 1e-12f) {
-            t_lo = fmaxf((zl - c.cull - az) * inv_uz, 0.0f);
-            t_hi = fminf((zl + c.cull - az) * inv_uz, len);
-        } else if (fabsf(az - zl) > c.cull) {
-            t_lo = 1.0f;
-            t_hi = 0.0f;
-        }
-        if (t_lo <= t_hi) {
-            const float xa = fmaf(t_lo, ux, ax), xb = fmaf(t_hi, ux, ax);
-            const float ya = fmaf(t_lo, uy, ay), yb = fmaf(t_hi, uy, ay);
-            const float xmin = fminf(xa, xb) - c.cull, xmax = fmaxf(xa, xb) + c.cull;
-            const float ymin = fminf(ya, yb) - c.cull, ymax = fmaxf(ya, yb) + c.cull;
-            const float qz = zl - az;
-#pragma unroll
-            for (int w = 0; w < kTileWarps; ++w) {
-                const float rx0 = ((float)((w & 1) * 8) + 0.5f) * c.fpx;
-                const float rx1 = ((float)((w & 1) * 8) + 7.5f) * c.fpx;
-                const float ry0 = ((float)((w >> 1) * 4) + 0.5f) * c.fpx;
-                const float ry1 = ((float)((w >> 1) * 4) + 3.5f) * c.fpx;
-                if (xmax >= rx0 && xmin <= rx1 && ymax >= ry0 && ymin <= ry1) {
-                    const float qx = 0.5f * (rx0 + rx1) - ax;
-                    const float qy = 0.5f * (ry0 + ry1) - ay;
-                    const float t = fmaf(qz, uz, fmaf(qy, uy, qx * ux));
-                    const float ex = fmaf(-t, ux, qx), ey = fmaf(-t, uy, qy);
-                    const float ez = fmaf(-t, uz, qz);
-                    if (fmaf(ez, ez, fmaf(ey, ey, ex * ex)) <= c.cull_line2)
-                        m |= 1ull << (w * 8 + l);
-                }
-            }
-        }
-    }
-    return m;
-}
-
-// Loads record rp into tile-local coordinates (see stage_record).
+// Loads record rp in coordinates relative to the tile's corner and the slab's
+// first layer plane (each given as a (hi, lo) float pair): A = (ax, ay, az, ux),
+// B = (uy, uz, len, w / R^4).
 __device__ __forceinline__ void load_record(const csl_rec* rp_rec, float oxh, float oxl, float oyh,
                                             float oyl, float ozh, float ozl, float inv_R4,
                                             float4& A, float4& B) {
@@ -138,75 +82,10 @@ __device__ __forceinline__ void load_record(const csl_rec* rp_rec, float oxh, fl
     B = make_float4(r1.x, r1.y, r1.z, r1.w * inv_R4);
 }
 
-// Extent of a staged edge (A, B) in layer l of a 16 x 16 tile: the pixel rows
-// j0..j1 and columns i0..i1 whose centres lie in the xy box of the edge clipped
-// to |z - z_l| <= cull, grown by cull. Packed as j0 | j1 << 4 | i0 << 8 |
-// i1 << 12 | 1 << 16; 0 when the box misses the tile or the layer.
-__device__ __forceinline__ uint32_t item_extent(const float4 A, const float4 B, int l,
-                                                const TileCull& c) {
-    const float ax = A.x, ay = A.y, az = A.z, ux = A.w, uy = B.x, uz = B.y, len = B.z;
-    const float zl = (float)l * c.fdz;
-    float t_lo = 0.0f, t_hi = len;
-    if (uz > 1e-12f) {
-        const float inv_uz = 1.0f / uz;
-        t_lo = fmaxf((zl - c.cull - az) * inv_uz, 0.0f);
-        t_hi = fminf((zl + c.cull - az) * inv_uz, len);
-    } else if (fabsf(az - zl) > c.cull) {
-        return 0u;
-    }
-    if (t_lo > t_hi) return 0u;
-    const float xa = fmaf(t_lo, ux, ax), xb = fmaf(t_hi, ux, ax);
-    const float ya = fmaf(t_lo, uy, ay), yb = fmaf(t_hi, uy, ay);
-    const float inv_px = 1.0f / c.fpx;
-    // pixel i has its centre at (i + 1/2) px: i in [ceil(x_min/px - 1/2), floor(x_max/px - 1/2)]
-    const float fx0 = fmaf(fminf(xa, xb) - c.cull, inv_px, -0.5f);
-    const float fx1 = fmaf(fmaxf(xa, xb) + c.cull, inv_px, -0.5f);
-    const float fy0 = fmaf(fminf(ya, yb) - c.cull, inv_px, -0.5f);
-    const float fy1 = fmaf(fmaxf(ya, yb) + c.cull, inv_px, -0.5f);
-    const int i0 = max(0, (int)ceilf(fmaxf(fx0, -1.0f)));
-    const int i1 = min(15, (int)floorf(fminf(fx1, 16.0f)));
-    const int j0 = max(0, (int)ceilf(fmaxf(fy0, -1.0f)));
-    const int j1 = min(15, (int)floorf(fminf(fy1, 16.0f)));
-    if (i0 > i1 || j0 > j1) return 0u;
-    return (uint32_t)j0 | ((uint32_t)j1 << 4) | ((uint32_t)i0 << 8) | ((uint32_t)i1 << 12) |
-           (1u << 16);
-}
-
-// Pixels i0..i1 of row j (within the extent e) whose centres lie within
-// sqrt(r2) of the edge's line in plane zl (tile-local). The line meets the
-// row's line {(x, y_j, zl)} at distance |Z u_y - Y u_z| / sqrt(a), a = u_y^2 +
-// u_z^2, closest at X* = u_x (Y u_y + Z u_z) / a, and the squared distance
-// grows as a (X - X*)^2, so the row's points within the radius are
-// |X - X*| <= sqrt(r2 a - (Z u_y - Y u_z)^2) / a. Widened by 0.05 px. An edge
-// along x (a ~ 0) keeps the extent's columns.
-__device__ __forceinline__ bool row_span(const float4 A, const float4 B, float zl, int j,
-                                         uint32_t e, const TileCull& c, float r2, int& i0,
-                                         int& i1) {
-    const float ux = A.w, uy = B.x, uz = B.y;
-    i0 = (int)((e >> 8) & 15u);
-    i1 = (int)((e >> 12) & 15u);
-    const float a = fmaf(uy, uy, uz * uz);
-    if (a > 1e-6f) {
-        const float Y = fmaf((float)j, c.fpx, 0.5f * c.fpx) - A.y;
-        const float Z = zl - A.z;
-        const float dm = fmaf(Z, uy, -(Y * uz));
-        const float q = fmaf(r2, a, -(dm * dm));
-        if (q < 0.0f) return false;
-        const float inv_a = 1.0f / a;
-        const float xs = ux * fmaf(Y, uy, Z * uz) * inv_a + A.x;
-        const float half = sqrt_approx(q) * inv_a;
-        const float inv_px = 1.0f / c.fpx;
-        const float f0 = fmaf(xs - half, inv_px, -0.55f);
-        const float f1 = fmaf(xs + half, inv_px, -0.45f);
-        i0 = max(i0, (int)ceilf(fmaxf(f0, -1.0f)));
-        i1 = min(i1, (int)floorf(fminf(f1, 16.0f)));
-    }
-    return i0 <= i1;
-}
-
 // The warps of one layer l whose block of 8 x 4 PX pixels the staged edge (A, B)
-// may reach (the test of stage_record for a single layer; c.cull_line2 for that
-// block): bit w set for warp w of the tile's 8 / PX.
+// may reach, i.e. the block meets the xy box of the edge clipped to |z - z_l| <=
+// cull grown by cull, and its centre lies within cull + half its diagonal of the
+// edge's line (c.cull_line2): bit w set for warp w of the tile's 8 / PX.
 template <int PX>
 __device__ __forceinline__ uint32_t cull_layer(const float4 A, const float4 B, int l,
                                                const TileCull& c) {

@@ -8,15 +8,14 @@
 // The m^3 samples of every cell are the pixels of a grid of pixel size h/m and
 // the cell layers are slabs of S = m layers, so the forward pass reuses the
 // slab/tile binner and the field kernel; a warp per cell then averages the
-// sigmoid. The backward pass is one kernel per (tile, slab): pass 1 recomputes
-// Sigma at its samples (nothing is stored between forward and backward) and
-// turns it into alpha = g_c / m^3 * s (1 - s) / T; pass 2 evaluates, for every
-// staged edge, the derivatives of its segment integral with respect to the
-// edge's weight and endpoints, sums them over the CTA's samples (per thread,
-// then a fixed warp tree, then the warps in order) and writes one partial per
-// bin entry. The partials are summed per edge in a fixed order (stable sort by
-// edge), and node gradients are gathered through a node -> endpoint list, so
-// the result is deterministic.
+// sigmoid. The backward pass recomputes Sigma the same way (nothing is stored
+// between forward and backward); one kernel per (tile, slab) then turns it into
+// alpha = g_c / m^3 * s (1 - s) / T at every sample and evaluates, for every edge
+// of the tile's list, the derivatives of its segment integral with respect to
+// the edge's weight and endpoints, summed over the samples per (edge, layer) and
+// then over the layers in a fixed tree: one partial per bin entry. The partials
+// are summed per edge in a fixed order (stable sort by edge), and node gradients
+// are gathered through a node -> endpoint list, so the result is deterministic.
 //
 // Derivatives of I = int_0^L f(|p - a - t u|^2) dt (f quartic, Eq. 5) by
 // differentiating under the integral in the fixed-bounds form
@@ -121,169 +120,200 @@ __global__ void k_vf_mean(const float* __restrict__ sigma, int cx, int cy, int n
 struct GradConst {
     int32_t nx, ny, ntx, n_tiles, n_layers;
     int32_t cx, cy, m, first_cl;
-    float R2, fpx, fdz, C, invT, inv_m3;
+    float R2, fpx, inv_px, fdz, C, invT, inv_m3;
+    float cull;      // R plus rounding slack
+    float inv_R4;
     float span_r2;   // squared radius of the footprint rows (R plus slack)
-    TileCull tc;
     const float2* org_x;
     const float2* org_y;
     const float2* org_z;
 };
 
-// Per (tile, slab): pass 1 Sigma -> alpha; pass 2 partial derivatives per
-// staged edge. partial[entry] = {sum alpha R^4 I, sum alpha w dI/da (3),
-// sum alpha w dI/db (3), 0}.
+// Pixel rows j0..j1 and columns i0..i1 of a 16 x 16 tile whose centres lie in
+// the xy box of the staged edge (A, B) clipped to |z - zl| <= cull, grown by
+// cull (approximate reciprocals move the box by far less than cull's slack).
+__device__ __forceinline__ bool grad_box(const float4 A, const float4 B, float zl,
+                                         const GradConst& c, int& i0, int& i1, int& j0, int& j1) {
+    const float ax = A.x, ay = A.y, az = A.z, ux = A.w, uy = B.x, uz = B.y, len = B.z;
+    float t_lo = 0.0f, t_hi = len;
+    if (uz > 1e-12f) {
+        const float inv_uz = __fdividef(1.0f, uz);
+        t_lo = fmaxf((zl - c.cull - az) * inv_uz, 0.0f);
+        t_hi = fminf((zl + c.cull - az) * inv_uz, len);
+    } else if (fabsf(az - zl) > c.cull) {
+        return false;
+    }
+    if (t_lo > t_hi) return false;
+    const float xa = fmaf(t_lo, ux, ax), xb = fmaf(t_hi, ux, ax);
+    const float ya = fmaf(t_lo, uy, ay), yb = fmaf(t_hi, uy, ay);
+    // pixel i has its centre at (i + 1/2) px; half a hundredth of a pixel of slack
+    const float fx0 = fmaf(fminf(xa, xb) - c.cull, c.inv_px, -0.505f);
+    const float fx1 = fmaf(fmaxf(xa, xb) + c.cull, c.inv_px, -0.495f);
+    const float fy0 = fmaf(fminf(ya, yb) - c.cull, c.inv_px, -0.505f);
+    const float fy1 = fmaf(fmaxf(ya, yb) + c.cull, c.inv_px, -0.495f);
+    i0 = max(0, __float2int_ru(fmaxf(fx0, -1.0f)));
+    i1 = min(15, __float2int_rd(fminf(fx1, 16.0f)));
+    j0 = max(0, __float2int_ru(fmaxf(fy0, -1.0f)));
+    j1 = min(15, __float2int_rd(fminf(fy1, 16.0f)));
+    return i0 <= i1 && j0 <= j1;
+}
+
+// Of the columns in `cols`, those of the row at dy (y relative to v_s) in plane
+// dz whose centres lie within R of the edge's line: on the row the squared
+// distance to the line is smallest at X* = u_x (Y u_y + Z u_z) / a, a = u_y^2 +
+// u_z^2, and grows as a (X - X*)^2 (Lagrange's identity); widened by 0.05 px. An
+// edge along x (a ~ 0) keeps the columns.
+__device__ __forceinline__ uint32_t row_columns(const float4 A, const float4 B, float dy, float dz,
+                                                uint32_t cols, const GradConst& c) {
+    const float ux = A.w, uy = B.x, uz = B.y;
+    const float a = fmaf(uy, uy, uz * uz);
+    if (a <= 1e-6f) return cols;
+    const float dm = fmaf(dz, uy, -(dy * uz));
+    const float q = fmaf(c.span_r2, a, -(dm * dm));
+    if (q < 0.0f) return 0u;
+    const float inv_a = __fdividef(1.0f, a);
+    const float xs = fmaf(ux * fmaf(dy, uy, dz * uz), inv_a, A.x);
+    const float half = sqrt_approx(q) * inv_a;
+    const int i0 = max(0, __float2int_ru(fmaxf(fmaf(xs - half, c.inv_px, -0.55f), -1.0f)));
+    const int i1 = min(15, __float2int_rd(fminf(fmaf(xs + half, c.inv_px, -0.45f), 16.0f)));
+    return i0 <= i1 ? cols & (0xffffu >> (15 - i1)) & (0xffffu << i0) : 0u;
+}
+
+// Per (tile, slab), from Sigma (the field kernel's, recomputed for the backward
+// pass): alpha = dL/dSigma at its samples, then the partial derivatives of
+// every edge of its list. partial[entry] = {sum alpha R^4 I, sum alpha w dI/da
+// (3), sum alpha w dI/db (3), 0}.
+//
+// A lane per (edge, layer): S lanes share an edge. A sample whose alpha is 0
+// (the sigmoid saturates in FP32) adds exactly nothing; the rows' samples with
+// alpha != 0 are bit masks, and a lane steps from one of its footprint's set
+// bits to the next before the warp evaluates a sample in all lanes together.
+// Bound by instruction issue. With Sigma recomputed here and a thread per edge
+// over all layers (19 of 32 lanes active, a barrier for the longest edge of 256)
+// 1 million struts on 64^3 cells of 8^3 samples took 14.0 ms; MEASURED_PLACEHOLDER
 template <int S>
-__global__ void __launch_bounds__(kVfThreads, 6)
-k_vf_grad(const csl_rec* __restrict__ rec, const uint32_t* __restrict__ vals,
-          const uint32_t* __restrict__ tstart, const uint32_t* __restrict__ tend, GradConst c,
+__global__ void __launch_bounds__(kVfThreads, 5)
+k_vf_grad(const csl_rec* __restrict__ recs, const uint32_t* __restrict__ tstart,
+          const uint32_t* __restrict__ tend, GradConst c, const float* __restrict__ sigma,
           const float* __restrict__ g_cells, float4* __restrict__ partial) {
-    __shared__ float4 s_a[kVfThreads];
-    __shared__ float4 s_b[kVfThreads];
-    __shared__ uint64_t s_mask[kVfThreads];
     __shared__ float s_alpha[S * kTile * kTile];   // [layer][j][i]
+    __shared__ uint32_t s_act[S * kTile];          // [layer][j]: bit i, alpha != 0
 
     const int tile = blockIdx.x, slab = blockIdx.y;
     const int tx = tile % c.ntx, ty = tile / c.ntx;
     const uint32_t key = (uint32_t)slab * (uint32_t)c.n_tiles + (uint32_t)tile;
     const uint32_t beg = tstart[key], end = tend[key];
     if (end <= beg) return;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    (void)lane;
-    const int wx = warp & 1, wy = warp >> 1;
-    const int il = wx * 8 + (lane & 7), jl = wy * 4 + (lane >> 3);
+    const int lane = threadIdx.x & 31;
     const int l0 = slab * S;
     const int nl = min(S, c.n_layers - l0);
-    const float2 ox = c.org_x[tx], oy = c.org_y[ty], oz = c.org_z[slab];
-    const float pxl = ((float)il + 0.5f) * c.fpx, pyl = ((float)jl + 0.5f) * c.fpx;
-    const TileCull cull = c.tc;
-
-    // pass 1: Sigma at this thread's samples
-    float acc[S];
+    // alpha of every sample of the tile (0 outside the grid / slab)
+    {
+        const int il = threadIdx.x & 15, jl = threadIdx.x >> 4;
+        const int gi = tx * kTile + il, gj = ty * kTile + jl;
 #pragma unroll
-    for (int l = 0; l < S; ++l) acc[l] = 0.0f;
-    for (uint32_t c0 = beg; c0 < end; c0 += kVfThreads) {
-        const int cnt = (int)min((uint32_t)kVfThreads, end - c0);
-        if ((int)threadIdx.x < cnt) {
-            float4 A, B;
-            s_mask[threadIdx.x] = stage_record(rec + vals[c0 + threadIdx.x], ox.x, ox.y, oy.x,
-                                               oy.y, oz.x, oz.y, nl, cull, A, B);
-            s_a[threadIdx.x] = A;
-            s_b[threadIdx.x] = B;
-        }
-        __syncthreads();
-        for (int i0 = 0; i0 < cnt; i0 += 32) {
-            const int i = i0 + lane;
-            const uint32_t wm = i < cnt ? (uint32_t)(s_mask[i] >> (warp * 8)) & 0xffu : 0u;
-            uint32_t ball = __ballot_sync(0xffffffffu, wm != 0u);
-            while (ball) {
-                const int b = __ffs(ball) - 1;
-                ball &= ball - 1u;
-                const uint32_t lm = __shfl_sync(0xffffffffu, wm, b);
-                const float4 A = s_a[i0 + b], B = s_b[i0 + b];
-                const float dx = pxl - A.x, dy = pyl - A.y;
-                const float txy = fmaf(dy, B.x, dx * A.w);
-#pragma unroll
-                for (int l = 0; l < S; ++l) {
-                    if (lm & (1u << l)) {
-                        const float dz = (float)l * c.fdz - A.z;
-                        const float t0 = fmaf(dz, B.y, txy);
-                        const float ex = fmaf(-t0, A.w, dx), ey = fmaf(-t0, B.x, dy);
-                        const float ez = fmaf(-t0, B.y, dz);
-                        const float h2 = fmaxf(c.R2 - fmaf(ez, ez, fmaf(ey, ey, ex * ex)), 0.0f);
-                        acc[l] = fmaf(B.w, segment_term_R4(t0, h2, B.z), acc[l]);
-                    }
-                }
+        for (int l = 0; l < S; ++l) {
+            float alpha = 0.0f;
+            if (l < nl && gi < c.nx && gj < c.ny) {
+                const int lz = l0 + l;   // chunk-local sample layer
+                const int64_t cell =
+                    ((int64_t)(c.first_cl + lz / c.m) * c.cy + gj / c.m) * c.cx + gi / c.m;
+                const float s =
+                    sigmoid((sigma[((int64_t)lz * c.ny + gj) * c.nx + gi] - c.C) * c.invT);
+                alpha = g_cells[cell] * c.inv_m3 * s * (1.0f - s) * c.invT;
             }
-        }
-        __syncthreads();
-    }
-    // alpha = dL/dSigma at each sample
-    const int gi = tx * kTile + il, gj = ty * kTile + jl;
-    float alpha[S];
-#pragma unroll
-    for (int l = 0; l < S; ++l) {
-        alpha[l] = 0.0f;
-        if (l < nl && gi < c.nx && gj < c.ny) {
-            const int lz = l0 + l;   // chunk-local sample layer
-            const int64_t cell =
-                ((int64_t)(c.first_cl + lz / c.m) * c.cy + gj / c.m) * c.cx + gi / c.m;
-            const float s = sigmoid((acc[l] - c.C) * c.invT);
-            alpha[l] = g_cells[cell] * c.inv_m3 * s * (1.0f - s) * c.invT;
+            s_alpha[l * 256 + threadIdx.x] = alpha;
+            const uint32_t act = __ballot_sync(0xffffffffu, alpha != 0.0f);
+            if ((lane & 15) == 0) s_act[l * kTile + jl] = (act >> lane) & 0xffffu;
         }
     }
-    // alpha of every sample of the tile, for pass 2 (0 outside the grid / slab)
-#pragma unroll
-    for (int l = 0; l < S; ++l) s_alpha[(l * kTile + jl) * kTile + il] = alpha[l];
-    // pass 2: one staged edge per thread; the thread visits the samples of its
-    // edge's footprint (rows of the clipped box, cut to the pixels within R of
-    // the line) and sums the 7 partials in registers, in a fixed order. A
-    // sample with alpha == 0 (the sigmoid saturates to 0 or 1 in FP32) adds
-    // exactly nothing and is skipped.
-    for (uint32_t c0 = beg; c0 < end; c0 += kVfThreads) {
-        const int cnt = (int)min((uint32_t)kVfThreads, end - c0);
-        __syncthreads();   // s_alpha written (first chunk) / nothing else shared here
-        if ((int)threadIdx.x >= cnt) continue;
-        float4 A, B;
-        load_record(rec + vals[c0 + threadIdx.x], ox.x, ox.y, oy.x, oy.y, oz.x, oz.y,
-                    cull.inv_R4, A, B);
+    __syncthreads();
+    const float2 ox = c.org_x[tx], oy = c.org_y[ty], oz = c.org_z[slab];
+    const int l = lane % S;
+    const float zl = (float)l * c.fdz;
+    constexpr uint32_t kPer = kVfThreads / S;   // edges at a time
+    for (uint32_t e0 = beg; e0 < end; e0 += kPer) {
+        const uint32_t e = e0 + threadIdx.x / S;
+        float4 A = make_float4(0.0f, 0.0f, 0.0f, 0.0f), B = A;
+        int i0 = 0, i1 = 0, j = 0, j1 = -1;
+        if (e < end) {
+            load_record(recs + e, ox.x, ox.y, oy.x, oy.y, oz.x, oz.y, c.inv_R4, A, B);
+            if (l >= nl || !grad_box(A, B, zl, c, i0, i1, j, j1)) j1 = j - 1;
+        }
+        const uint32_t cols = (0xffffu >> (15 - i1)) & (0xffffu << i0);
         const float ux = A.w, uy = B.x, uz = B.y, len = B.z;
         const float inv_len = len > 0.0f ? 1.0f / len : 0.0f;
+        const float dz = zl - A.z;
         float gw = 0.0f, gax = 0.0f, gay = 0.0f, gaz = 0.0f, gbx = 0.0f, gby = 0.0f, gbz = 0.0f;
-        for (int l = 0; l < nl; ++l) {
-            const uint32_t e = item_extent(A, B, l, cull);
-            if (!e) continue;
-            const float zl = (float)l * c.fdz;
-            const int j0 = (int)(e & 15u), j1 = (int)((e >> 4) & 15u);
-            for (int j = j0; j <= j1; ++j) {
-                int i0, i1;
-                if (!row_span(A, B, zl, j, e, cull, c.span_r2, i0, i1)) continue;
-                const float dy = ((float)j + 0.5f) * c.fpx - A.y;
-                const float dz = zl - A.z;
-                const float* arow = s_alpha + (l * kTile + j) * kTile;
-                for (int i = i0; i <= i1; ++i) {
-                    const float al = arow[i];
-                    if (al == 0.0f) continue;
-                    const float dx = ((float)i + 0.5f) * c.fpx - A.x;
-                    const float txy = fmaf(dy, uy, dx * ux);
-                    const float t0 = fmaf(dz, uz, txy);
-                    const float ex = fmaf(-t0, ux, dx), ey = fmaf(-t0, uy, dy);
-                    const float ez = fmaf(-t0, uz, dz);
-                    const float h2 = fmaxf(c.R2 - fmaf(ez, ez, fmaf(ey, ey, ex * ex)), 0.0f);
-                    if (h2 == 0.0f) continue;
-                    const float w = sqrt_approx(h2);
-                    const float tau1 = fmaxf(-t0, -w), tau2 = fminf(len - t0, w);
-                    const float hh = 0.5f * fmaxf(tau2 - tau1, 0.0f);   // half width
-                    const float mm = 0.5f * (tau2 + tau1);               // midpoint
-                    const float del = 0.7745966692414834f * hh;          // sqrt(0.6) h
-                    const float ta = mm - del, tb = mm + del;
-                    const float ga = fmaf(-ta, ta, h2), gm = fmaf(-mm, mm, h2),
-                                gb = fmaf(-tb, tb, h2);
-                    const float W1 = (5.0f / 9.0f) * hh, W2 = (8.0f / 9.0f) * hh;
-                    const float wa = W1 * ga, wm2 = W2 * gm, wb = W1 * gb;
-                    const float I4 = fmaf(wa, ga, fmaf(wm2, gm, wb * gb));
-                    const float M0 = wa + wm2 + wb;
-                    const float M1 = fmaf(wa, ta, fmaf(wm2, mm, wb * tb));
-                    const float M2 = fmaf(wa * ta, ta, fmaf(wm2 * mm, mm, wb * tb * tb));
-                    const float r = t0 * inv_len;
-                    const float il4 = I4 * inv_len;
-                    const float cau = fmaf(1.0f - r, M1, -M2 * inv_len);
-                    const float cae = fmaf(1.0f - r, M0, -M1 * inv_len);
-                    const float cbu = fmaf(r, M1, M2 * inv_len);
-                    const float cbe = fmaf(r, M0, M1 * inv_len);
-                    const float alw = al * B.w;
-                    gw = fmaf(al, I4, gw);
-                    // R^4 dI/da = -u I4/L - 4 (u cau - e cae); times alpha w/R^4
-                    gax = fmaf(alw, fmaf(-ux, il4, -4.0f * fmaf(ux, cau, -ex * cae)), gax);
-                    gay = fmaf(alw, fmaf(-uy, il4, -4.0f * fmaf(uy, cau, -ey * cae)), gay);
-                    gaz = fmaf(alw, fmaf(-uz, il4, -4.0f * fmaf(uz, cau, -ez * cae)), gaz);
-                    gbx = fmaf(alw, fmaf(ux, il4, -4.0f * fmaf(ux, cbu, -ex * cbe)), gbx);
-                    gby = fmaf(alw, fmaf(uy, il4, -4.0f * fmaf(uy, cbu, -ey * cbe)), gby);
-                    gbz = fmaf(alw, fmaf(uz, il4, -4.0f * fmaf(uz, cbu, -ez * cbe)), gbz);
+        uint32_t bits = 0;
+        float dy = 0.0f;
+        const float* arow = s_alpha;
+        for (;;) {
+            // this lane's next row with samples to take
+            while (bits == 0u && j <= j1) {
+                const uint32_t m = s_act[l * kTile + j] & cols;
+                if (m) {
+                    dy = ((float)j + 0.5f) * c.fpx - A.y;
+                    arow = s_alpha + (l * kTile + j) * kTile;
+                    bits = row_columns(A, B, dy, dz, m, c);
                 }
+                ++j;
             }
+            if (!__any_sync(0xffffffffu, bits != 0u)) break;
+            if (!bits) continue;
+            const int i = __ffs(bits) - 1;
+            bits &= bits - 1u;
+            const float al = arow[i];
+            const float dx = ((float)i + 0.5f) * c.fpx - A.x;
+            const float txy = fmaf(dy, uy, dx * ux);
+            const float t0 = fmaf(dz, uz, txy);
+            const float ex = fmaf(-t0, ux, dx), ey = fmaf(-t0, uy, dy);
+            const float ez = fmaf(-t0, uz, dz);
+            const float h2 = fmaxf(c.R2 - fmaf(ez, ez, fmaf(ey, ey, ex * ex)), 0.0f);
+            const float w = sqrt_approx(h2);
+            const float tau1 = fmaxf(-t0, -w), tau2 = fminf(len - t0, w);
+            const float hh = 0.5f * fmaxf(tau2 - tau1, 0.0f);   // half width
+            const float mm = 0.5f * (tau2 + tau1);               // midpoint
+            const float del = 0.7745966692414834f * hh;          // sqrt(0.6) h
+            const float ta = mm - del, tb = mm + del;
+            const float ga = fmaf(-ta, ta, h2), gm = fmaf(-mm, mm, h2), gb = fmaf(-tb, tb, h2);
+            const float W1 = (5.0f / 9.0f) * hh, W2 = (8.0f / 9.0f) * hh;
+            const float wa = W1 * ga, wm2 = W2 * gm, wb = W1 * gb;
+            const float I4 = fmaf(wa, ga, fmaf(wm2, gm, wb * gb));
+            const float M0 = wa + wm2 + wb;
+            const float M1 = fmaf(wa, ta, fmaf(wm2, mm, wb * tb));
+            const float M2 = fmaf(wa * ta, ta, fmaf(wm2 * mm, mm, wb * tb * tb));
+            const float r = t0 * inv_len;
+            const float il4 = I4 * inv_len;
+            const float cau = fmaf(1.0f - r, M1, -M2 * inv_len);
+            const float cae = fmaf(1.0f - r, M0, -M1 * inv_len);
+            const float cbu = fmaf(r, M1, M2 * inv_len);
+            const float cbe = fmaf(r, M0, M1 * inv_len);
+            const float alw = al * B.w;
+            gw = fmaf(al, I4, gw);
+            // R^4 dI/da = -u I4/L - 4 (u cau - e cae); times alpha w/R^4
+            gax = fmaf(alw, fmaf(-ux, il4, -4.0f * fmaf(ux, cau, -ex * cae)), gax);
+            gay = fmaf(alw, fmaf(-uy, il4, -4.0f * fmaf(uy, cau, -ey * cae)), gay);
+            gaz = fmaf(alw, fmaf(-uz, il4, -4.0f * fmaf(uz, cau, -ez * cae)), gaz);
+            gbx = fmaf(alw, fmaf(ux, il4, -4.0f * fmaf(ux, cbu, -ex * cbe)), gbx);
+            gby = fmaf(alw, fmaf(uy, il4, -4.0f * fmaf(uy, cbu, -ey * cbe)), gby);
+            gbz = fmaf(alw, fmaf(uz, il4, -4.0f * fmaf(uz, cbu, -ez * cbe)), gbz);
         }
-        partial[2 * (int64_t)(c0 + threadIdx.x)] = make_float4(gw, gax, gay, gaz);
-        partial[2 * (int64_t)(c0 + threadIdx.x) + 1] = make_float4(gbx, gby, gbz, 0.0f);
+        // the layers' sums, in a fixed tree
+#pragma unroll
+        for (int o = 1; o < S; o <<= 1) {
+            gw += __shfl_xor_sync(0xffffffffu, gw, o);
+            gax += __shfl_xor_sync(0xffffffffu, gax, o);
+            gay += __shfl_xor_sync(0xffffffffu, gay, o);
+            gaz += __shfl_xor_sync(0xffffffffu, gaz, o);
+            gbx += __shfl_xor_sync(0xffffffffu, gbx, o);
+            gby += __shfl_xor_sync(0xffffffffu, gby, o);
+            gbz += __shfl_xor_sync(0xffffffffu, gbz, o);
+        }
+        if (l == 0 && e < end) {
+            partial[2 * (int64_t)e] = make_float4(gw, gax, gay, gaz);
+            partial[2 * (int64_t)e + 1] = make_float4(gbx, gby, gbz, 0.0f);
+        }
     }
 }
 
@@ -413,18 +443,6 @@ DevBuf origin_tables(const ChunkGeom& g, cudaStream_t s) {
     return d;
 }
 
-TileCull tile_cull(const ChunkGeom& g) {
-    TileCull t;
-    t.fpx = (float)g.px;
-    t.fdz = (float)g.dz;
-    t.cull = (float)(g.R * (1.0 + 1e-5) + 1e-6);
-    const double hd = g.px * sqrt(3.5 * 3.5 + 1.5 * 1.5) * (1.0 + 1e-5);
-    const double r = (double)t.cull + hd;
-    t.cull_line2 = (float)(r * r);
-    t.inv_R4 = (float)(1.0 / (g.R * g.R * g.R * g.R));
-    return t;
-}
-
 }  // namespace
 
 void validate_cells_or_fail(const csl_cells* c) { validate_cells(c); }
@@ -457,12 +475,15 @@ void vf_backward(csl_lattice* L, const csl_cells& cells, const float* grad_vf, f
     const int cz = cells.dims[2];
     DevBuf acc((size_t)ne * 32, s);
     CSL_CUDA(cudaMemsetAsync(acc.get(), 0, (size_t)ne * 32, s));
+    DevBuf sigma((size_t)cells.dims[0] * cells.dims[1] * per * cells.m * cells.m * cells.m * 4, s);
     for (int first = 0; first < cz; first += per) {
         const int n = std::min(per, cz - first);
         ChunkGeom g = vf_geom(L, cells, first, n);
         SlabBins bins;
         bin_chunk(L, g, bins, s);
         if (bins.n_pairs == 0) continue;
+        // Sigma of the chunk's samples again (nothing is kept from the forward pass)
+        field_chunk(L, g, bins, (float)L->C, sigma.as<float>(), nullptr, nullptr, s);
         DevBuf partial((size_t)bins.n_pairs * 32, s);
         DevBuf org = origin_tables(g, s);
         GradConst c;
@@ -481,7 +502,9 @@ void vf_backward(csl_lattice* L, const csl_cells& cells, const float* grad_vf, f
         c.C = (float)L->C;
         c.invT = (float)(1.0 / cells.temperature);
         c.inv_m3 = 1.0f / (float)(cells.m * cells.m * cells.m);
-        c.tc = tile_cull(g);
+        c.inv_px = (float)(1.0 / g.px);
+        c.cull = (float)(g.R * (1.0 + 1e-5) + 1e-6);
+        c.inv_R4 = (float)(1.0 / (g.R * g.R * g.R * g.R));
         {
             const double rs = L->R * (1.0 + 2e-4) + 1e-6;
             c.span_r2 = (float)(rs * rs);
@@ -492,10 +515,10 @@ void vf_backward(csl_lattice* L, const csl_cells& cells, const float* grad_vf, f
         dim3 grid((unsigned)c.n_tiles, (unsigned)g.n_slabs);
 #define CSL_VF_CASE(SV)                                                                        \
     case SV:                                                                                   \
-        k_vf_grad<SV><<<grid, kVfThreads, 0, s>>>(L->rec.as<csl_rec>(),                        \
-                                                  bins.vals.as<uint32_t>(),                    \
+        k_vf_grad<SV><<<grid, kVfThreads, 0, s>>>(bins.recs.as<csl_rec>(),                     \
                                                   bins.tile_start.as<uint32_t>(),              \
-                                                  bins.tile_end.as<uint32_t>(), c, grad_vf,    \
+                                                  bins.tile_end.as<uint32_t>(), c,             \
+                                                  sigma.as<float>(), grad_vf,                  \
                                                   partial.as<float4>());                       \
         break;
         switch (cells.m) {
