@@ -331,7 +331,7 @@ void csl_contours_free(csl_contours* c) {
     if (c->on_device) {   // arrays grown in place (slicing) go back through their registry
         for (void* p : {(void*)c->layer_loop_off, (void*)c->loop_vert_off, (void*)c->xy,
                         (void*)c->edge_id})
-            if (p && !growmap_free(p)) cudaFree(p);
+            if (p && !growmap_free(p)) result_free(p);
     } else {
         host_block_free(c->layer_loop_off);   // offsets block
         host_block_free(c->xy);               // vertex block (edge ids included)
@@ -391,10 +391,7 @@ csl_status csl_contours_create(int32_t n_layers, int64_t n_loops, int64_t n_vert
         c->n_loops = n_loops;
         c->n_verts = n_verts;
         auto up = [&](void** dst, const void* src, size_t bytes) {
-            if (cudaMalloc(dst, bytes ? bytes : 16) != cudaSuccess) {
-                cudaGetLastError();
-                fail(CSL_ERR_OOM, "device allocation of the contours failed");
-            }
+            *dst = result_alloc(bytes, s, "device allocation of the contours failed");
             if (bytes) CSL_CUDA(cudaMemcpyAsync(*dst, src, bytes, cudaMemcpyHostToDevice, s));
         };
         up((void**)&c->layer_loop_off, layer_loop_off, (size_t)(n_layers + 1) * 8);
@@ -933,10 +930,12 @@ csl_status csl_slice_layers(csl_lattice* L, const csl_slice_desc* desc, void* st
             c->on_device = 1;
             c->n_loops = n_loops;
             c->n_verts = n_verts;
-            if (cudaMalloc((void**)&c->layer_loop_off, (size_t)(d.n_layers + 1) * 8) != cudaSuccess) {
-                cudaGetLastError();
+            try {
+                c->layer_loop_off = (int64_t*)result_alloc(
+                    (size_t)(d.n_layers + 1) * 8, s, "device allocation of the contours failed");
+            } catch (...) {
                 delete c;
-                fail(CSL_ERR_OOM, "device allocation of the contours failed");
+                throw;
             }
             int layer = 0;
             for (auto& cc : dev_chunks) {   // rebased already; entry 0 repeats the last end
@@ -961,10 +960,11 @@ csl_status csl_slice_layers(csl_lattice* L, const csl_slice_desc* desc, void* st
             c->n_loops = n_loops;
             c->n_verts = n_verts;
             auto dst_alloc = [&](void** p, size_t b) {
-                if (cudaMalloc(p, b ? b : 16) != cudaSuccess) {
-                    cudaGetLastError();
+                try {
+                    *p = result_alloc(b, s, "device allocation of the contours failed");
+                } catch (...) {
                     csl_contours_free(c);
-                    fail(CSL_ERR_OOM, "device allocation of the contours failed");
+                    throw;
                 }
             };
             dst_alloc((void**)&c->layer_loop_off, (size_t)(d.n_layers + 1) * 8);

@@ -495,10 +495,7 @@ csl_status csl_batch_contours(const csl_batch* b, int32_t job, int32_t dst_on_de
         }
         try {
             auto alloc = [&](void** p, size_t bytes) {
-                if (cudaMalloc(p, bytes ? bytes : 16) != cudaSuccess) {
-                    cudaGetLastError();
-                    fail(CSL_ERR_OOM, "device allocation of the contours failed");
-                }
+                *p = result_alloc(bytes, b->st, "device allocation of the contours failed");
             };
             if (on_dev) {
                 alloc((void**)&c->layer_loop_off, nl * 8);

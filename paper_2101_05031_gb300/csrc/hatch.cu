@@ -275,10 +275,7 @@ csl_status csl_hatch_layers(const csl_contours* ct, double y0, double spacing, i
         h->n_segments = n_seg;
         auto alloc = [&](void** p, size_t b) {
             if (dst_on_device) {
-                if (cudaMalloc(p, b ? b : 16) != cudaSuccess) {
-                    cudaGetLastError();
-                    fail(CSL_ERR_OOM, "device allocation of the hatches failed");
-                }
+                *p = result_alloc(b, s, "device allocation of the hatches failed");
             } else {
                 *p = host_block_alloc(b ? b : 16);
             }
@@ -357,8 +354,8 @@ csl_status csl_hatch_layers(const csl_contours* ct, double y0, double spacing, i
 void csl_hatches_free(csl_hatches* h) {
     if (!h) return;
     if (h->on_device) {
-        cudaFree(h->layer_seg_off);
-        cudaFree(h->seg);
+        result_free(h->layer_seg_off);
+        result_free(h->seg);
     } else {
         host_block_free(h->layer_seg_off);
         host_block_free(h->seg);

@@ -223,10 +223,7 @@ extern "C" csl_status csl_simplify_contours(const csl_contours* in, int32_t nx, 
         c->on_device = 1;
         c->n_loops = n_loops;
         auto dst_alloc = [&](void** p, size_t bytes) {
-            if (cudaMalloc(p, bytes ? bytes : 16) != cudaSuccess) {
-                cudaGetLastError();
-                fail(CSL_ERR_OOM, "device allocation of the contours failed");
-            }
+            *p = result_alloc(bytes, s, "device allocation of the contours failed");
         };
         dst_alloc((void**)&c->layer_loop_off, (size_t)(n_layers + 1) * 8);
         dst_alloc((void**)&c->loop_vert_off, (size_t)(n_loops + 1) * 8);
