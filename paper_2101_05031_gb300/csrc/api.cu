@@ -568,8 +568,10 @@ csl_status csl_slice_layers(csl_lattice* L, const csl_slice_desc* desc, void* st
             int64_t copied = 0;       // vertices already copied (chunks 0..k)
             cudaStream_t cs = nullptr;
             cudaEvent_t ev = nullptr;
+            cudaStream_t chunk_stream = nullptr;   // where the copies run without cs
             ~Spec() {
                 if (cs) cudaStreamSynchronize(cs);
+                else if (block) cudaStreamSynchronize(chunk_stream);   // left by an error
                 if (ev) cudaEventDestroy(ev);
                 if (cs) cudaStreamDestroy(cs);
                 if (block) host_block_free(block);
@@ -577,14 +579,16 @@ csl_status csl_slice_layers(csl_lattice* L, const csl_slice_desc* desc, void* st
         } spec;
         if (want_contours && !on_dev && d.n_layers > 0) {
             spec.block = host_block_take_largest(&spec.bytes);
+            spec.chunk_stream = s;
             if (spec.block) {
                 spec.eid_off = vertex_block_eid_offset(spec.bytes, want_eid);
                 spec.cap = want_eid ? std::min<int64_t>(spec.eid_off / 8,
                                                         (spec.bytes - spec.eid_off) / 4)
                                     : (int64_t)(spec.bytes / 8);
                 // with a budget the copies run on the chunk's stream (its
-                // buffers are freed right after, in stream order)
-                if (!budgeted) {
+                // buffers are freed right after, in stream order); a single
+                // chunk has nothing to overlap them with
+                if (!budgeted && n_chunks > 1) {
                     CSL_CUDA(cudaStreamCreateWithFlags(&spec.cs, cudaStreamNonBlocking));
                     CSL_CUDA(cudaEventCreateWithFlags(&spec.ev, cudaEventDisableTiming));
                 }
@@ -636,15 +640,18 @@ csl_status csl_slice_layers(csl_lattice* L, const csl_slice_desc* desc, void* st
             if (budgeted) {   // to_host() copies this chunk
             } else if (spec_all && spec.copied + cc.n_verts <= spec.cap) {
                 if (cc.n_verts) {
-                    CSL_CUDA(cudaEventRecord(spec.ev, ks));
-                    CSL_CUDA(cudaStreamWaitEvent(spec.cs, spec.ev, 0));
+                    cudaStream_t copy = spec.cs ? spec.cs : ks;
+                    if (spec.cs) {
+                        CSL_CUDA(cudaEventRecord(spec.ev, ks));
+                        CSL_CUDA(cudaStreamWaitEvent(spec.cs, spec.ev, 0));
+                    }
                     char* base = static_cast<char*>(spec.block);
                     CSL_CUDA(cudaMemcpyAsync(base + spec.copied * 8, cc.xy.get(), cc.n_verts * 8,
-                                             cudaMemcpyDeviceToHost, spec.cs));
+                                             cudaMemcpyDeviceToHost, copy));
                     if (want_eid)
                         CSL_CUDA(cudaMemcpyAsync(base + spec.eid_off + spec.copied * 4,
                                                  cc.eid.get(), cc.n_verts * 4,
-                                                 cudaMemcpyDeviceToHost, spec.cs));
+                                                 cudaMemcpyDeviceToHost, copy));
                 }
                 spec.copied += cc.n_verts;
             } else {

@@ -478,6 +478,10 @@ __global__ void k_jump_rank(const uint32_t* __restrict__ dist, const uint32_t* _
     if (__syncthreads_or(live) && threadIdx.x == 0) done[it] = 1u;
 }
 
+// Chunks of at most this many splitters resolve their long cycles before the
+// host knows how many there are.
+constexpr int64_t kAheadSplitters = (int64_t)1 << 17;
+
 // Splitter cycles of at most kShortCycle splitters (all the small loops) are
 // resolved by walking them; the rest go to pointer jumping on a compact list.
 constexpr int kShortCycle = 16;
@@ -582,6 +586,89 @@ __global__ void k_long_ranks(const uint32_t* __restrict__ lcm, const uint32_t* _
         cm[t] = lcm[u];
         rank_start[t] = dist[hu] - dist[u];
         if (hu == (uint32_t)u) loop_len[t] = dist[u];
+    }
+}
+
+// The whole resolution of the long cycles by one block, for at most kLongBlock
+// of their splitters: the cycle minima by doubling, the break before each head,
+// the ranks by doubling, back to splitter order, as the kernels above do it
+// over the grid, with the links in shared memory. One launch instead of 2 log2
+// + 4 (each step then costs a launch of about 3 us whatever the count: 22 of
+// them for the 2,000 long-cycle splitters of a 200^2 x 50 slice). Does nothing
+// where there are more.
+constexpr int kLongBlock = 12288;
+constexpr int kLongThreads = 1024;
+
+__global__ void __launch_bounds__(kLongThreads)
+k_long_block(const uint32_t* __restrict__ n_long, const uint32_t* __restrict__ long_list,
+             const uint32_t* __restrict__ long_pos, const uint32_t* __restrict__ split_id,
+             const uint32_t* __restrict__ seg_next, const uint32_t* __restrict__ seg_len,
+             const uint32_t* __restrict__ spos, int64_t ns, int64_t cap,
+             uint32_t* __restrict__ cm, uint32_t* __restrict__ rank_start,
+             uint32_t* __restrict__ loop_len) {
+    extern __shared__ uint32_t s_link[];
+    const uint32_t count = *n_long;
+    if (count == 0u || count > (uint32_t)kLongBlock) return;
+    // (a replay whose sizes changed, flagged, may count more than its list holds)
+    const uint32_t nl = (uint32_t)min((int64_t)count, cap);
+    uint32_t *a = s_link, *an = a + nl, *b = an + nl, *bn = b + nl;
+    for (uint32_t u = threadIdx.x; u < nl; u += kLongThreads) {
+        const uint32_t t = long_list[u];
+        const uint32_t nu = long_pos[seg_next[t]];
+        a[u] = split_id[t];
+        an[u] = nu < nl ? nu : u;   // out of range only in a flagged replay
+    }
+    __syncthreads();
+    for (int it = 0; it < 32; ++it) {   // cycle minimum; done when a step changes nothing
+        bool changed = false;
+        for (uint32_t u = threadIdx.x; u < nl; u += kLongThreads) {
+            const uint32_t x = a[u], nt = an[u];
+            const uint32_t m = min(x, a[nt]);
+            changed |= m != x;
+            b[u] = m;
+            bn[u] = an[nt];
+        }
+        const bool more = __syncthreads_or(changed);
+        uint32_t* t = a; a = b; b = t;
+        t = an; an = bn; bn = t;
+        if (!more) break;
+    }
+    // a: the minima. The cycles broken before their heads: an = next, b = distance
+    for (uint32_t u = threadIdx.x; u < nl; u += kLongThreads) {
+        const uint32_t t = long_list[u];
+        const uint32_t nt = seg_next[t];
+        const uint32_t nu = long_pos[nt];
+        an[u] = (nu >= nl || a[nu] == split_id[nt]) ? kNil : nu;
+        b[u] = seg_len[t];
+        cm[t] = a[u];
+    }
+    __syncthreads();
+    uint32_t *d = b, *d2 = a;   // the minima are in cm from here on
+    for (int it = 0; it < 32; ++it) {   // distance to the end of the broken cycle
+        bool live = false;
+        for (uint32_t u = threadIdx.x; u < nl; u += kLongThreads) {
+            const uint32_t nt = an[u];
+            if (nt >= nl) {
+                d2[u] = d[u];
+                bn[u] = nt;
+            } else {
+                d2[u] = d[u] + d[nt];
+                bn[u] = an[nt];
+                live |= an[nt] < nl;
+            }
+        }
+        const bool more = __syncthreads_or(live);
+        uint32_t* t = d; d = d2; d2 = t;
+        t = an; an = bn; bn = t;
+        if (!more) break;
+    }
+    for (uint32_t u = threadIdx.x; u < nl; u += kLongThreads) {
+        const uint32_t t = long_list[u];
+        const uint32_t sp = spos[cm[t]];
+        uint32_t hu = (int64_t)sp < ns ? long_pos[sp] : kNil;
+        if (hu >= nl) hu = u;   // only in a flagged replay
+        rank_start[t] = d[hu] - d[u];
+        if (hu == u) loop_len[t] = d[u];
     }
 }
 
@@ -706,12 +793,14 @@ void contours_chunk(const ChunkGeom& g, double C, const float* sigma, const uint
     // 32-bit crossing ids: fewer than 2^27 edge words keeps every count below 2^32
     if (n_words >= ((int64_t)1 << 27)) fail(CSL_ERR_CAPACITY, "marching squares: chunk too large");
 
-    // small: [0] status, [1] crossings, [2] splitters, [3..66] done, [67] long count
+    // small: [0] status, [1] crossings, [2] splitters, [3..66] done, [67] long
+    // count, [68, 69] loops << 32 | crossings they cover
     DevBuf small(4 * 80, s);
     CSL_CUDA(cudaMemsetAsync(small.get(), 0, 4 * 80, s));
     uint32_t* status = small.as<uint32_t>();
     uint32_t* done = small.as<uint32_t>() + 3;
     uint32_t* n_long = small.as<uint32_t>() + 67;
+    int64_t* tot = reinterpret_cast<int64_t*>(small.as<uint32_t>() + 68);
     uint32_t* flag = rp ? rp->flag : status;   // where replay mismatches go
 
     DevBuf ew((size_t)n_words * 4, s), prefix((size_t)n_words * 4, s);
@@ -831,18 +920,34 @@ void contours_chunk(const ChunkGeom& g, double C, const float* sigma, const uint
                                       long_list.as<uint32_t>(), long_pos.as<uint32_t>(), n_long,
                                       rank_start.as<uint32_t>(), loop_len.as<uint32_t>());
     CSL_LAUNCH_CHECK("ms short cycles");
-    int64_t nl;
+    // Long cycles: by one block where they fit. A small chunk does not read
+    // their count first (a read-back takes as long as the block): it is read
+    // with the loop count below, and only if the block could not take them do
+    // the grid's kernels run, and the numbering of the loops again.
+    const bool ahead = !replay && ns <= kAheadSplitters;
+    auto long_block = [&] {
+        const int smem = 4 * 4 * (int)std::min<int64_t>(ns, kLongBlock);
+        CSL_CUDA(cudaFuncSetAttribute(k_long_block, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      4 * 4 * kLongBlock));
+        k_long_block<<<1, kLongThreads, smem, s>>>(
+            n_long, long_list.as<uint32_t>(), long_pos.as<uint32_t>(), split_id.as<uint32_t>(),
+            seg_next.as<uint32_t>(), seg_len.as<uint32_t>(), spos.as<uint32_t>(), ns, ns,
+            cm.as<uint32_t>(), rank_start.as<uint32_t>(), loop_len.as<uint32_t>());
+        CSL_LAUNCH_CHECK("ms long cycles");
+    };
+    int64_t nl = 0;
     if (replay) {
         nl = rp->plan->nl;
         k_check_u32<<<1, 32, 0, s>>>(n_long, (uint32_t)nl, flag);
         CSL_LAUNCH_CHECK("check long cycles");
-    } else {
+    } else if (!ahead) {
         uint32_t v = 0;
         read_to_host(&v, n_long, 4, s);
         nl = v;
         if (rp) rp->plan->nl = nl;
     }
-    if (nl > 0) {
+    if (ahead || (nl > 0 && nl <= kLongBlock)) long_block();
+    auto long_grid = [&] {
         // cycle minimum by doubling (later steps copy the converged result forward)
         int max_it = 1;
         while (((int64_t)1 << max_it) < nl + 1) ++max_it;
@@ -885,22 +990,35 @@ void contours_chunk(const ChunkGeom& g, double C, const float* sigma, const uint
                                         cm.as<uint32_t>(), rank_start.as<uint32_t>(),
                                         loop_len.as<uint32_t>());
         CSL_LAUNCH_CHECK("ms long ranks");
-    }
-    DevBuf packed((size_t)ns * 8, s), scan((size_t)ns * 8, s), tot(8, s);
-    k_head_flags<<<gs, 256, 0, s>>>(cm.as<uint32_t>(), split_id.as<uint32_t>(),
-                                    loop_len.as<uint32_t>(), ns, packed.as<int64_t>());
-    CSL_LAUNCH_CHECK("ms heads");
-    exclusive_scan_i64(packed.as<int64_t>(), scan.as<int64_t>(), ns, tot.as<int64_t>(), s);
+    };
+    if (nl > kLongBlock) long_grid();
+    DevBuf packed((size_t)ns * 8, s), scan((size_t)ns * 8, s);
+    auto number_loops = [&] {
+        k_head_flags<<<gs, 256, 0, s>>>(cm.as<uint32_t>(), split_id.as<uint32_t>(),
+                                        loop_len.as<uint32_t>(), ns, packed.as<int64_t>());
+        CSL_LAUNCH_CHECK("ms heads");
+        exclusive_scan_i64(packed.as<int64_t>(), scan.as<int64_t>(), ns, tot, s);
+    };
+    number_loops();
     int64_t n_loops;
     if (replay) {
         n_loops = rp->plan->n_loops;
-        k_check_packed<<<1, 32, 0, s>>>(tot.as<int64_t>(), n_loops, n_cross, status, flag);
+        k_check_packed<<<1, 32, 0, s>>>(tot, n_loops, n_cross, status, flag);
         CSL_LAUNCH_CHECK("check loops");
     } else {
-        const int64_t packed_total = read_i64(tot.as<int64_t>(), s);
-        uint32_t st = 0;
-        read_to_host(&st, status, 4, s);
-        if (st) fail(CSL_ERR_CUDA, "marching squares: inconsistent successor links");
+        uint32_t h[70];
+        read_to_host(h, small.get(), sizeof h, s);
+        if (ahead) {
+            nl = h[67];
+            if (rp) rp->plan->nl = nl;
+            if (nl > kLongBlock) {
+                long_grid();
+                number_loops();
+                read_to_host(h, small.get(), sizeof h, s);
+            }
+        }
+        if (h[0]) fail(CSL_ERR_CUDA, "marching squares: inconsistent successor links");
+        const int64_t packed_total = (int64_t)(((uint64_t)h[69] << 32) | h[68]);
         n_loops = packed_total >> 32;
         if ((packed_total & 0xffffffffLL) != n_cross)
             fail(CSL_ERR_CUDA, "marching squares: loops do not cover every crossing");
