@@ -20,8 +20,8 @@
 //      the mean of the 4 corner values is >= C, i.e. each entry turns to the
 //      next side, else to the previous one. Inside lies on the left.
 //   4. the head of a loop is its smallest id, which is a local minimum
-//      (pred > id < succ). Splitters = all local minima plus a hashed 1-in-32
-//      sample of crossings; each splitter walks its segment to the next
+//      (pred > id < succ). Splitters = all local minima plus a hashed sample
+//      of crossings; each splitter walks its segment to the next
 //      splitter, so no thread walks a whole long loop;
 //   5. on the graph of splitters (one cycle per loop), a cycle of at most 16
 //      splitters (every small loop) is resolved by walking it; on the rest,
@@ -317,10 +317,18 @@ __global__ void __launch_bounds__(256, 6) k_emit(const float* __restrict__ sigma
 }
 
 // Splitters cut every loop into short segments: every local minimum
-// (pred > id < succ; the loop's smallest id is one) and a hashed 1-in-32
-// sample, so that a smooth loop with a single local minimum is cut too.
-__device__ __forceinline__ bool is_splitter(uint32_t i, uint32_t pred_i, uint32_t succ_i) {
-    return (pred_i > i && succ_i > i) || ((i * 2654435761u) >> 27) == 0u;
+// (pred > id < succ; the loop's smallest id is one) and a hashed sample of one
+// in 2^bits, so that a smooth loop with a single local minimum is cut too.
+__device__ __forceinline__ bool is_splitter(uint32_t i, uint32_t pred_i, uint32_t succ_i,
+                                            int bits) {
+    return (pred_i > i && succ_i > i) || ((i * 2654435761u) >> (32 - bits)) == 0u;
+}
+// 1 in 32; in small chunks 1 in 8 or 16, because there the longest walk is what
+// the segment kernels take (one 2000^2 layer: 15 + 24 us at 1 in 32, 5 + 9 us at
+// 1 in 8; 200^2 x 50: 35 + 33 us and, at 1 in 16, 10 + 13 us), and the splitters
+// more are few enough for the block that resolves long cycles.
+int splitter_bits(int64_t n_cross) {
+    return n_cross <= ((int64_t)1 << 16) ? 3 : (n_cross <= ((int64_t)1 << 18) ? 4 : 5);
 }
 
 // For the successor s of every crossing i (i is s's predecessor): nxt[s] =
@@ -332,7 +340,7 @@ __device__ __forceinline__ bool is_splitter(uint32_t i, uint32_t pred_i, uint32_
 // somebody's successor (the entry crossing of its exit cell), so every entry
 // is written; in a replay whose sizes changed, entries left out keep the 0
 // they were cleared to (no splitter).
-__global__ void k_split_flags(const Xing* __restrict__ rec, int64_t n,
+__global__ void k_split_flags(const Xing* __restrict__ rec, int64_t n, int bits,
                               uint32_t* __restrict__ nxt, uint32_t* status) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x) {
@@ -342,7 +350,7 @@ __global__ void k_split_flags(const Xing* __restrict__ rec, int64_t n,
             continue;
         }
         const uint32_t sc = rec[q].succ;
-        const bool sp = is_splitter(q, (uint32_t)i, sc);
+        const bool sp = is_splitter(q, (uint32_t)i, sc, bits);
         nxt[q] = (sc & 0x7fffffffu) | (sp ? 0x80000000u : 0u);
     }
 }
@@ -482,18 +490,19 @@ __global__ void k_jump_rank(const uint32_t* __restrict__ dist, const uint32_t* _
 // host knows how many there are.
 constexpr int64_t kAheadSplitters = (int64_t)1 << 17;
 
-// Splitter cycles of at most kShortCycle splitters (all the small loops) are
+// Splitter cycles of at most short_cycle splitters (all the small loops) are
 // resolved by walking them; the rest go to pointer jumping on a compact list.
-constexpr int kShortCycle = 16;
+// 16, or 32 where splitter_bits samples more densely.
+int short_cycle_of(int64_t n_cross) { return splitter_bits(n_cross) < 5 ? 32 : 16; }
 constexpr uint32_t kNil = 0xffffffffu;
 
 // cm[t] = the cycle's smallest splitter id when t's cycle closes within
-// kShortCycle steps; otherwise t is appended to the long list. The head of a
+// short_cycle steps; otherwise t is appended to the long list. The head of a
 // short cycle (the splitter holding its smallest id) then walks it once more:
 // rank_start = crossings of the loop before each segment, loop_len at the head.
 __global__ void k_short_cycles(const uint32_t* __restrict__ split_id,
                                const uint32_t* __restrict__ seg_next,
-                               const uint32_t* __restrict__ seg_len, int64_t ns,
+                               const uint32_t* __restrict__ seg_len, int64_t ns, int short_cycle,
                                uint32_t* __restrict__ cm, uint32_t* __restrict__ long_list,
                                uint32_t* __restrict__ long_pos, uint32_t* __restrict__ n_long,
                                uint32_t* __restrict__ rank_start,
@@ -506,7 +515,7 @@ __global__ void k_short_cycles(const uint32_t* __restrict__ split_id,
         if (t < ns) {
             uint32_t v = seg_next[t], mn = split_id[t];
             int n = 1;
-            while (v != (uint32_t)t && n < kShortCycle) {
+            while (v != (uint32_t)t && n < short_cycle) {
                 const uint32_t id = split_id[v];
                 mn = id < mn ? id : mn;
                 v = seg_next[v];
@@ -522,7 +531,7 @@ __global__ void k_short_cycles(const uint32_t* __restrict__ split_id,
                     rank_start[w] = acc;
                     acc += seg_len[w];
                     w = seg_next[w];
-                } while (w != (uint32_t)t && ++m < kShortCycle);
+                } while (w != (uint32_t)t && ++m < short_cycle);
                 loop_len[t] = acc;
             }
         }
@@ -883,7 +892,8 @@ void contours_chunk(const ChunkGeom& g, double C, const float* sigma, const uint
     // changed may leave some out: there they start as 0 (no splitter)
     if (rp) CSL_CUDA(cudaMemsetAsync(nxt.get(), 0, (size_t)n_cross * 4, s));
     const unsigned gx = grid_for(n_cross, 256);
-    k_split_flags<<<gx, 256, 0, s>>>(rec.as<Xing>(), n_cross, nxt.as<uint32_t>(), status);
+    k_split_flags<<<gx, 256, 0, s>>>(rec.as<Xing>(), n_cross, splitter_bits(n_cross),
+                                     nxt.as<uint32_t>(), status);
     CSL_LAUNCH_CHECK("ms splitter flags");
     // the list's room: every crossing, or a replay's planned count
     const int64_t ns_cap = replay ? rp->plan->ns : n_cross;
@@ -916,8 +926,8 @@ void contours_chunk(const ChunkGeom& g, double C, const float* sigma, const uint
     DevBuf rank_start((size_t)ns * 4, s), loop_len((size_t)ns * 4, s);
     if (replay) CSL_CUDA(cudaMemsetAsync(long_list.get(), 0, (size_t)ns * 4, s));
     k_short_cycles<<<gs, 256, 0, s>>>(split_id.as<uint32_t>(), seg_next.as<uint32_t>(),
-                                      seg_len.as<uint32_t>(), ns, cm.as<uint32_t>(),
-                                      long_list.as<uint32_t>(), long_pos.as<uint32_t>(), n_long,
+                                      seg_len.as<uint32_t>(), ns, short_cycle_of(n_cross),
+                                      cm.as<uint32_t>(), long_list.as<uint32_t>(), long_pos.as<uint32_t>(), n_long,
                                       rank_start.as<uint32_t>(), loop_len.as<uint32_t>());
     CSL_LAUNCH_CHECK("ms short cycles");
     // Long cycles: by one block where they fit. A small chunk does not read
