@@ -11,14 +11,14 @@
 //      32-bit edge words per mask word;
 //   2. a prefix sum of the edge words' popcounts numbers the crossings in
 //      (layer, edge id) order: id = prefix[word] + popc(lower bits);
-//   3. k_emit: per mask word, only the cells with a crossing side: the vertex
-//      on each of the cell's own two edges (the zero of the linear interpolant
-//      of Sigma - C) and, for each side where a contour enters the cell, its
-//      successor. Walking the sides counter-clockwise, a side from an inside
-//      to an outside corner is an entry, from outside to inside an exit; a
-//      saddle (two inside corners on a diagonal) joins its inside corners when
-//      the mean of the 4 corner values is >= C, i.e. each entry turns to the
-//      next side, else to the previous one. Inside lies on the left.
+//   3. k_emit: per crossing, its vertex (the zero of the linear interpolant of
+//      Sigma - C) and the crossings before and after it, each the other
+//      crossing side of one of the two cells that share the edge. Walking a
+//      cell's sides counter-clockwise, a side from an inside to an outside
+//      corner is an entry, from outside to inside an exit; a saddle (two
+//      inside corners on a diagonal) joins its inside corners when the mean of
+//      the 4 corner values is >= C, i.e. each entry turns to the next side,
+//      else to the previous one. Inside lies on the left.
 //   4. the head of a loop is its smallest id, which is a local minimum
 //      (pred > id < succ). Splitters = all local minima plus a hashed sample
 //      of crossings; each splitter walks its segment to the next
@@ -30,8 +30,8 @@
 //      gives every segment its distance from the head;
 //   6. a prefix sum over the heads (loop length) numbers the loops in head
 //      order and places them; every splitter writes its segment there.
-// Crossings are 16-byte records {x, y, successor, edge id}, so one walk step
-// is one load.
+// Vertices, edge ids (where asked for) and successors lie in arrays of their
+// own: a walk follows the 4-byte successors alone.
 #include <math.h>
 
 #include <algorithm>
@@ -49,12 +49,6 @@ struct MsConst {
     int64_t edge_wpl;     // edge words per layer
     int32_t n_layers;
     float C, fx0, fy0, fpx;
-};
-
-struct __align__(16) Xing {
-    float x, y;
-    uint32_t succ;
-    int32_t eid;
 };
 
 __device__ __forceinline__ uint32_t spread16(uint32_t x) {
@@ -130,199 +124,23 @@ __device__ __forceinline__ float2 fused_vertex(const FusedIn& F, const Dense& D,
 }
 
 
-// A block of k_emit covers a band of kEmitRows cell rows and kEmitWords mask
-// words (32 cells each) of one layer: one thread per (row, word). The Sigma
-// values its vertices and saddles need (pixel rows J0 - 1 .. J0 + kEmitRows - 1,
-// columns 32 k0 - 1 .. 32 (k0 + kEmitWords) - 1) are staged into shared memory
-// first with coalesced loads, so that every Sigma row is read from DRAM about
-// once instead of as scattered words at each crossing. A staged row has a
-// pitch of kEmitPitch floats: pixel 32 k0 + c sits at column 4 + c (16-byte
-// aligned, so a thread moves 4 pixels with one vector load and store), pixel
-// 32 k0 - 1 at column 3.
-constexpr int kEmitRows = 8, kEmitWords = 32;
-constexpr int kEmitPitch = 32 * kEmitWords + 4;
-static_assert(32 * kEmitWords == 4 * 256, "one 4-pixel vector per thread and row");
-
-// grid: x over (band of kEmitRows rows J <= ny, segment of kEmitWords mask
-// words), y = layer. FUSED: vertices and saddle decisions from the fused pass
-// (F) instead of Sigma.
-template <bool FUSED>
-__global__ void __launch_bounds__(256, 6) k_emit(const float* __restrict__ sigma, const uint32_t* __restrict__ mask,
-                       MsConst c, Dense D, FusedIn F, Xing* __restrict__ rec, uint32_t n_cap,
-                       uint32_t* flag) {
-    __shared__ __align__(16) float s_sig[FUSED ? 4 : (kEmitRows + 1) * kEmitPitch];
-    const int layer = blockIdx.y;
-    const int n_segs = (c.mwr + kEmitWords - 1) / kEmitWords;
-    const int band = blockIdx.x / n_segs, seg = blockIdx.x - band * n_segs;
-    const int J0 = band * kEmitRows, k0 = seg * kEmitWords;
-    const int J = J0 + (int)(threadIdx.x / kEmitWords), k = k0 + (int)(threadIdx.x % kEmitWords);
-    const uint32_t* m = mask + (int64_t)layer * c.mask_wpl;
-    const float* sg = FUSED ? nullptr : sigma + (int64_t)layer * c.nx * c.ny;
-    // this thread's mask words, edge words and prefix sums (of its row, the
-    // next word and the row above), loaded before the staging so that their
-    // latency overlaps it; the other prefixes follow from these
-    const bool live = J <= c.ny && k < c.mwr;
-    const bool last = k + 1 >= c.mwr;
-    uint32_t in0 = 0u, in1 = 0u, up = 0u, up1 = 0u;
-    uint32_t e0 = 0u, e1 = 0u, e2 = 0u, p0 = 0u, u0 = 0u, u1 = 0u, q0 = 0u;
-    if (live) {
-        in0 = m[(int64_t)J * c.mwr + k];
-        in1 = last ? 0u : m[(int64_t)J * c.mwr + k + 1];
-        up = m[(int64_t)(J + 1) * c.mwr + k];          // J + 1 <= ny + 1 < H
-        up1 = last ? 0u : m[(int64_t)(J + 1) * c.mwr + k + 1];
-        const int64_t wb = layer * D.edge_wpl + (int64_t)J * D.ewr + 2 * k;
-        const int64_t wu = wb + D.ewr;
-        e0 = D.ew[wb];
-        e1 = D.ew[wb + 1];
-        e2 = last ? 0u : D.ew[wb + 2];
-        p0 = D.prefix[wb];
-        u0 = D.ew[wu];
-        u1 = D.ew[wu + 1];
-        q0 = D.prefix[wu];
-    }
-    if (!FUSED) {   // pixel (i, j) -> s_sig[(j - (J0 - 1)) * kEmitPitch + 4 + i - 32 k0]
-        const int ib = 32 * k0 + 4 * (int)threadIdx.x;   // this thread's 4 pixels of each row
-        // whole vectors need 16-byte aligned rows (nx % 4 == 0) and 4 pixels inside
-        const bool vec = (c.nx & 3) == 0 && (reinterpret_cast<uintptr_t>(sg) & 15) == 0 &&
-                         ib + 3 < c.nx;
-#pragma unroll
-        for (int r = 0; r < kEmitRows + 1; ++r) {
-            const int j = J0 - 1 + r;
-            float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-            if (j >= 0 && j < c.ny) {
-                const float* row = sg + (int64_t)j * c.nx;
-                if (vec) {
-                    v = __ldg(reinterpret_cast<const float4*>(row + ib));
-                } else {
-                    if (ib < c.nx) v.x = row[ib];
-                    if (ib + 1 < c.nx) v.y = row[ib + 1];
-                    if (ib + 2 < c.nx) v.z = row[ib + 2];
-                    if (ib + 3 < c.nx) v.w = row[ib + 3];
-                }
-                if (threadIdx.x == 0)   // the pixel left of the band (column 3)
-                    s_sig[r * kEmitPitch + 3] = (k0 > 0 && 32 * k0 - 1 < c.nx) ? row[32 * k0 - 1]
-                                                                              : 0.0f;
-            } else if (threadIdx.x == 0) {
-                s_sig[r * kEmitPitch + 3] = 0.0f;
-            }
-            *reinterpret_cast<float4*>(&s_sig[r * kEmitPitch + 4 + 4 * threadIdx.x]) = v;
-        }
-        __syncthreads();
-    }
-    // Sigma at padded sample (I, J) of this block (0 outside the grid, like the ring)
-    auto value_s = [&](int I, int J2) -> float {
-        return s_sig[(J2 - J0) * kEmitPitch + (I - 32 * k0) + 3];
-    };
-    if (!live) return;
-    const uint32_t hb = in0 ^ ((in0 >> 1) | (in1 << 31));          // bottom side of cell I
-    const uint32_t vb = in0 ^ up;                                  // left side
-    const uint32_t vr = (vb >> 1) | ((in1 ^ up1) << 31);           // right side
-    const uint32_t ht = up ^ ((up >> 1) | (up1 << 31));            // top side
-    uint32_t active = hb | vb | vr | ht;
-    if (!active) return;
-    // the prefix of a word is its left neighbour's plus that word's crossings:
-    // every crossing id below comes from registers
-    const uint32_t p1 = p0 + __popc(e0), p2 = last ? 0u : p1 + __popc(e1);
-    const uint32_t q1 = q0 + __popc(u0);
-    while (active) {
-        const int b = __ffs(active) - 1;
-        active &= active - 1u;
-        const int I = 32 * k + b;
-        // corners counter-clockwise: 0 (I,J), 1 (I+1,J), 2 (I+1,J+1), 3 (I,J+1)
-        const uint32_t in_c0 = (in0 >> b) & 1u, in_c3 = (up >> b) & 1u;
-        const uint32_t in_c1 = b < 31 ? (in0 >> (b + 1)) & 1u : in1 & 1u;
-        const uint32_t in_c2 = b < 31 ? (up >> (b + 1)) & 1u : up1 & 1u;
-        // ids of the crossings on the cell's sides (valid where the side crosses):
-        // in the interleaved edge words, sample si's h edge is bit 2 (si % 16) and
-        // its v edge the next bit; the right side is sample b + 1's v edge, the
-        // top side the h edge of sample b in the row above
-        const int bit = 2 * (b & 15);
-        const uint32_t eb_w = b < 16 ? e0 : e1, pb_w = b < 16 ? p0 : p1;
-        const uint32_t id_bottom = pb_w + __popc(eb_w & ((1u << bit) - 1u));
-        const uint32_t id_left = id_bottom + ((eb_w >> bit) & 1u);
-        const int sr = b + 1, bit_r = 2 * (sr & 15) + 1;
-        const uint32_t er_w = sr < 16 ? e0 : (sr < 32 ? e1 : e2);
-        const uint32_t pr_w = sr < 16 ? p0 : (sr < 32 ? p1 : p2);
-        const uint32_t id_right = pr_w + __popc(er_w & ((1u << bit_r) - 1u));
-        const uint32_t id_top = (b < 16 ? q0 : q1) + __popc((b < 16 ? u0 : u1) & ((1u << bit) - 1u));
-        auto side = [&](int sd) -> uint32_t {   // sides: 0 bottom, 1 right, 2 top, 3 left
-            return sd == 0 ? id_bottom : (sd == 1 ? id_right : (sd == 2 ? id_top : id_left));
-        };
-        const bool h_own = (hb >> b) & 1u, v_own = (vb >> b) & 1u;
-        // Sigma only where a vertex is placed (or a saddle is decided)
-        const float v0 = (!FUSED && (h_own || v_own)) ? value_s(I, J) : 0.0f;
-        const int64_t eb = 2 * ((int64_t)J * c.W + I);
-        if (h_own) {   // vertex on the bottom edge (I, J) -> (I+1, J)
-            const uint32_t id = id_bottom;
-            if (id >= n_cap) { atomicOr(flag, 1u); continue; }
-            float2 xy;
-            if (FUSED) {
-                xy = fused_vertex(F, D, layer, I, J, 0);
-            } else {
-                const float v1 = value_s(I + 1, J);
-                const float sa = in_c0 ? v0 : v1, sbv = in_c0 ? v1 : v0;
-                const float t = __fdividef(sa - c.C, sa - sbv);   // in [0, 1]; sa > C > sbv
-                const float xp = in_c0 ? ((float)I - 0.5f + t) : ((float)I + 0.5f - t);
-                xy = make_float2(c.fx0 + xp * c.fpx, c.fy0 + ((float)J - 0.5f) * c.fpx);
-            }
-            *reinterpret_cast<float2*>(&rec[id].x) = xy;
-            rec[id].eid = (int32_t)eb;
-        }
-        if (v_own) {   // vertex on the left edge (I, J) -> (I, J+1)
-            const uint32_t id = id_left;
-            if (id >= n_cap) { atomicOr(flag, 1u); continue; }
-            float2 xy;
-            if (FUSED) {
-                xy = fused_vertex(F, D, layer, I, J, 1);
-            } else {
-                const float v3 = value_s(I, J + 1);
-                const float sa = in_c0 ? v0 : v3, sbv = in_c0 ? v3 : v0;
-                const float t = __fdividef(sa - c.C, sa - sbv);   // in [0, 1]; sa > C > sbv
-                const float yp = in_c0 ? ((float)J - 0.5f + t) : ((float)J + 0.5f - t);
-                xy = make_float2(c.fx0 + ((float)I - 0.5f) * c.fpx, c.fy0 + yp * c.fpx);
-            }
-            *reinterpret_cast<float2*>(&rec[id].x) = xy;
-            rec[id].eid = (int32_t)(eb + 1);
-        }
-        // successors. Side k runs from corner k to corner k+1; bit k of nxt is corner k+1.
-        const uint32_t cs = in_c0 | (in_c1 << 1) | (in_c2 << 2) | (in_c3 << 3);
-        const uint32_t nxt = ((cs >> 1) | (cs << 3)) & 0xfu;
-        const uint32_t enter = cs & ~nxt & 0xfu;   // inside -> outside
-        const uint32_t leave = ~cs & nxt & 0xfu;   // outside -> inside
-        if (__popc(enter) == 1) {
-            const uint32_t a = side(__ffs(enter) - 1);
-            if (a < n_cap) rec[a].succ = side(__ffs(leave) - 1);
-            else atomicOr(flag, 1u);
-        } else if (enter) {
-            bool joined;
-            if (FUSED) {
-                const uint32_t sw = F.saddle[(int64_t)layer * c.mask_wpl + (int64_t)J * c.mwr +
-                                             (I >> 5)];
-                joined = (sw >> (I & 31)) & 1u;
-            } else {
-                const float w0 = value_s(I, J), w1 = value_s(I + 1, J);
-                const float w2 = value_s(I + 1, J + 1), w3 = value_s(I, J + 1);
-                joined = 0.25f * (w0 + w1 + w2 + w3) >= c.C;
-            }
-            const int k0 = __ffs(enter) - 1, k1 = 31 - __clz(enter);
-            const uint32_t a0 = side(k0), a1 = side(k1);
-            if (a0 < n_cap && a1 < n_cap) {
-                rec[a0].succ = side(joined ? ((k0 + 1) & 3) : ((k0 + 3) & 3));
-                rec[a1].succ = side(joined ? ((k1 + 1) & 3) : ((k1 + 3) & 3));
-            } else {
-                atomicOr(flag, 1u);
-            }
-        }
-    }
-}
+// A block of k_emit covers a band of kEmitRows sample rows and kEmitWords mask
+// words (32 samples each) of one layer, a warp per row at a time. A lane takes a
+// crossing: it computes the vertex and, from the two cells that share the
+// edge, the crossings before and after it on the contour, so that records and
+// successors are written whole and in order, and the splitters are known here.
+// The crossings of a warp's row are listed in shared memory first (ids are
+// consecutive along a row), which keeps every lane busy; edge words and their
+// prefix sums of the band and of one row and one word around it are staged as
+// pairs {word, prefix}. Sigma is read where a crossing needs it (through L1):
+// a tile of it in shared memory costs a barrier and half the warps.
+constexpr int kEmitRows = 8, kEmitWords = 32, kEmitWarps = 4;
+constexpr int kEmitList = 512;                     // crossings listed at a time per warp
+constexpr int kEmitPitch = 2 * kEmitWords + 2;     // edge words 2 k0 - 1 .. 2 (k0 + kEmitWords)
 
 // Splitters cut every loop into short segments: every local minimum
 // (pred > id < succ; the loop's smallest id is one) and a hashed sample of one
-// in 2^bits, so that a smooth loop with a single local minimum is cut too.
-__device__ __forceinline__ bool is_splitter(uint32_t i, uint32_t pred_i, uint32_t succ_i,
-                                            int bits) {
-    return (pred_i > i && succ_i > i) || ((i * 2654435761u) >> (32 - bits)) == 0u;
-}
+// in 2^bits, so that a smooth loop with a single local minimum is cut too:
 // 1 in 32; in small chunks 1 in 8 or 16, because there the longest walk is what
 // the segment kernels take (one 2000^2 layer: 15 + 24 us at 1 in 32, 5 + 9 us at
 // 1 in 8; 200^2 x 50: 35 + 33 us and, at 1 in 16, 10 + 13 us), and the splitters
@@ -331,27 +149,159 @@ int splitter_bits(int64_t n_cross) {
     return n_cross <= ((int64_t)1 << 16) ? 3 : (n_cross <= ((int64_t)1 << 18) ? 4 : 5);
 }
 
-// For the successor s of every crossing i (i is s's predecessor): nxt[s] =
-// succ(s) | (s is a splitter) << 31, the only array the segment walks read
-// and the one whose top bits number the splitters. Thread i reads its own
-// successor and its successor's (records of one contour lie close together),
-// so no separate predecessor array is built. A successor out of range is
-// reported through *status and nothing is written for it. Every crossing is
-// somebody's successor (the entry crossing of its exit cell), so every entry
-// is written; in a replay whose sizes changed, entries left out keep the 0
-// they were cleared to (no splitter).
-__global__ void k_split_flags(const Xing* __restrict__ rec, int64_t n, int bits,
-                              uint32_t* __restrict__ nxt, uint32_t* status) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const uint32_t q = rec[i].succ;
-        if ((int64_t)q >= n) {
-            atomicOr(status, ST_CAPACITY);
-            continue;
+// grid: x over (band of kEmitRows rows J <= ny, segment of kEmitWords mask
+// words), y = layer. FUSED: vertices and saddle decisions from the fused pass
+// (F) instead of Sigma. nxt[i] = succ(i) | (i is a splitter) << 31, the only
+// array the segment walks read and the one whose top bits number the
+// splitters. 389 million crossings of 500 layers of 2000^2: 3.55 ms, bound by
+// issue (about 200 instructions per crossing); a thread per mask word stepping
+// through its cells, with a Sigma tile in shared memory and 16-byte records
+// written in parts, took 6.9 ms and the splitters 1.5 ms more (19 of 32 lanes
+// active). 8 warps per block 4.3 ms, 16 rows per block 4.3, 4 rows 3.9.
+template <bool FUSED>
+__global__ void __launch_bounds__(32 * kEmitWarps, 12) k_emit(
+    const float* __restrict__ sigma, const uint32_t* __restrict__ mask, MsConst c, Dense D,
+    FusedIn F, int bits, float2* __restrict__ oxy, int32_t* __restrict__ oeid,
+    uint32_t* __restrict__ nxt, uint32_t n_cap, uint32_t* flag) {
+    __shared__ uint2 s_e[(kEmitRows + 2) * kEmitPitch];   // row J0 - 1 + r, word 2 k0 - 1 + x
+    __shared__ uint32_t s_in[kEmitRows * kEmitWords];
+    __shared__ uint16_t s_list[kEmitWarps * kEmitList];   // edge word << 5 | bit
+    const int layer = blockIdx.y;
+    const int n_segs = (c.mwr + kEmitWords - 1) / kEmitWords;
+    const int band = blockIdx.x / n_segs, seg = blockIdx.x - band * n_segs;
+    const int J0 = band * kEmitRows, k0 = seg * kEmitWords;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t* m = mask + (int64_t)layer * c.mask_wpl;
+    const float* sg = FUSED ? nullptr : sigma + (int64_t)layer * c.nx * c.ny;
+    const int64_t ebase = layer * D.edge_wpl;
+#pragma unroll
+    for (int x = threadIdx.x; x < (kEmitRows + 2) * kEmitPitch; x += 32 * kEmitWarps) {
+        const int r = x / kEmitPitch, w = 2 * k0 - 1 + (x - r * kEmitPitch), Jr = J0 - 1 + r;
+        uint2 v = make_uint2(0u, 0u);
+        if (Jr >= 0 && Jr < c.H && w >= 0 && w < D.ewr) {
+            const int64_t at = ebase + (int64_t)Jr * D.ewr + w;
+            v = make_uint2(D.ew[at], D.prefix[at]);
         }
-        const uint32_t sc = rec[q].succ;
-        const bool sp = is_splitter(q, (uint32_t)i, sc, bits);
-        nxt[q] = (sc & 0x7fffffffu) | (sp ? 0x80000000u : 0u);
+        s_e[x] = v;
+    }
+#pragma unroll
+    for (int r = warp; r < kEmitRows; r += kEmitWarps)
+        s_in[r * kEmitWords + lane] = J0 + r < c.H && k0 + lane < c.mwr
+                                          ? m[(int64_t)(J0 + r) * c.mwr + k0 + lane]
+                                          : 0u;
+    __syncthreads();
+
+    // Sigma at padded sample (I, J) (0 outside the grid, like the ring)
+    auto value = [&](int I, int J) -> float {
+        return (uint32_t)(I - 1) < (uint32_t)c.nx && (uint32_t)(J - 1) < (uint32_t)c.ny
+                   ? __ldg(sg + (int64_t)(J - 1) * c.nx + (I - 1))
+                   : 0.0f;
+    };
+    // saddle cell (I, J): its inside corners are joined
+    auto joined = [&](int I, int J) -> bool {
+        if (FUSED) {
+            const uint32_t sw =
+                F.saddle[(int64_t)layer * c.mask_wpl + (int64_t)J * c.mwr + (I >> 5)];
+            return (sw >> (I & 31)) & 1u;
+        }
+        const float w0 = value(I, J), w1 = value(I + 1, J);
+        const float w2 = value(I + 1, J + 1), w3 = value(I, J + 1);
+        return 0.25f * (w0 + w1 + w2 + w3) >= c.C;
+    };
+
+    uint16_t* list = s_list + warp * kEmitList;
+    for (int wr = warp; wr < kEmitRows; wr += kEmitWarps) {
+        const int J = J0 + wr;
+        const uint2* er = s_e + (wr + 1) * kEmitPitch + 1;   // row J from word 2 k0
+        const uint2 ea = er[2 * lane], eb = er[2 * lane + 1];
+        // the row's crossings in this segment: ids first .. first + n - 1 (words past
+        // the end of the row hold no crossings)
+        const uint32_t first = er[0].y;
+        const int n = (int)__reduce_add_sync(0xffffffffu, __popc(ea.x) + __popc(eb.x));
+        // Sigma of row J where it is inside the grid, and of the row after it
+        const bool row0 = (uint32_t)(J - 1) < (uint32_t)c.ny, row1 = (uint32_t)J < (uint32_t)c.ny;
+        const float* srow = FUSED ? nullptr : sg + ((int64_t)(J - 1) * c.nx + 32 * k0 - 1);
+        const int eid0 = (int)(2 * ((int64_t)J * c.W + 32 * k0));
+        for (int base = 0; base < n; base += kEmitList) {
+            __syncwarp();
+#pragma unroll
+            for (int half = 0; half < 2; ++half) {
+                uint32_t bitsw = half ? eb.x : ea.x;
+                int at = (int)((half ? eb.y : ea.y) - first) - base;
+                const int code = (2 * lane + half) << 5;
+                for (; bitsw; bitsw &= bitsw - 1u, ++at)
+                    if ((uint32_t)at < (uint32_t)kEmitList)
+                        list[at] = (uint16_t)(code | (__ffs(bitsw) - 1));
+            }
+            __syncwarp();
+            const int room = min(kEmitList, n - base);
+            for (int t = lane; t < room; t += 32) {
+                const int e = list[t], dir = e & 1, il = e >> 1, I = 32 * k0 + il;
+                const uint32_t id = first + (uint32_t)(base + t);
+                const bool in0 = (s_in[wr * kEmitWords + (il >> 5)] >> (il & 31)) & 1u;
+                // The contour enters cell (I, J) where inside lies on its left, else the
+                // cell on the other side of the edge, through side `own` (0 bottom, 1
+                // right, 2 top, 3 left). Its successor is the other crossing side; in a
+                // saddle cell the side after `own` if joined, else the one before.
+                const bool here = in0 != (dir != 0);
+                const int cl = il - (here ? 0 : dir), down = here ? 0 : 1 - dir;
+                const int own = here ? 3 * dir : 2 - dir;
+                const uint2* cw = er - down * kEmitPitch + (cl >> 4);
+                const uint2 lo = cw[0], up = cw[kEmitPitch];
+                const uint2 ri = er[((cl + 1) >> 4) - down * kEmitPitch];
+                const int sh = 2 * cl & 31, sr = (2 * cl + 2 & 31) + 1;
+                const uint32_t hv = lo.x >> sh;
+                const uint32_t others = ((hv & 1u) | (((ri.x >> sr) & 1u) << 1) |
+                                         (((up.x >> sh) & 1u) << 2) | ((hv & 2u) << 2)) &
+                                        ~(1u << own);
+                int side = 31 - __clz(others);
+                if (others & (others - 1u))
+                    side = (own + (joined(32 * k0 + cl, J - down) ? 1 : 3)) & 3;
+                const uint2 sw = side == 2 ? up : (side == 1 ? ri : lo);
+                const int sbit = side == 1 ? sr : sh + (side == 3);
+                const uint32_t succ = sw.y + __popc(sw.x & ((1u << sbit) - 1u));
+                // Ids order edges by row and, in a row, by column, so a local minimum is
+                // an edge (I, J) -> (I, J+1) (of the cell below an edge (I, J) -> (I+1, J)
+                // every other side comes first) that is joined to the top side of the
+                // cell on its left and not to the bottom side of the one on its right.
+                const uint2* lw = er + ((il - 1) >> 4);
+                const int sl = 2 * il - 2 & 31;
+                bool lowest = dir && ((lw[kEmitPitch].x >> sl) & 1u);
+                if (lowest) {
+                    if (((lw[0].x >> sl) & 3u) == 3u) lowest = joined(I - 1, J) != here;
+                    if ((er[il >> 4].x >> (2 * il & 31)) & 1u) {   // bottom, or a saddle
+                        const uint32_t rv = er[(il + 1) >> 4].x >> ((2 * il + 2 & 31) + 1);
+                        const uint32_t rt = er[kEmitPitch + (il >> 4)].x >> (2 * il & 31);
+                        lowest = lowest && (rv & rt & 1u) && joined(I, J) != here;
+                    }
+                }
+                if (max(id, succ) >= n_cap) {
+                    atomicOr(flag, 1u);
+                    continue;
+                }
+                float2 xy;
+                if (FUSED) {
+                    xy = fused_vertex(F, D, layer, I, J, dir);
+                } else {
+                    const bool in_x = (uint32_t)(I - 1) < (uint32_t)c.nx;
+                    const bool nx_x = dir ? in_x : (uint32_t)I < (uint32_t)c.nx;
+                    const float v0 = in_x && row0 ? __ldg(srow + il) : 0.0f;
+                    const float v1 = nx_x && (dir ? row1 : row0)
+                                         ? __ldg(srow + (il + (dir ? c.nx : 1)))
+                                         : 0.0f;
+                    const float sa = in0 ? v0 : v1, sb = in0 ? v1 : v0;
+                    const float tt = __fdividef(sa - c.C, sa - sb);   // in [0, 1]; sa > C > sb
+                    const float p0 = (float)(dir ? J : I);
+                    const float p = in0 ? (p0 - 0.5f + tt) : (p0 + 0.5f - tt);
+                    xy = dir ? make_float2(c.fx0 + ((float)I - 0.5f) * c.fpx, c.fy0 + p * c.fpx)
+                             : make_float2(c.fx0 + p * c.fpx, c.fy0 + ((float)J - 0.5f) * c.fpx);
+                }
+                oxy[id] = xy;
+                if (oeid) oeid[id] = eid0 + e;
+                const bool sampled = ((id * 2654435761u) >> (32 - bits)) == 0u;
+                nxt[id] = succ | (lowest || sampled ? 0x80000000u : 0u);
+            }
+        }
     }
 }
 
@@ -701,59 +651,66 @@ __global__ void k_check_packed(const int64_t* __restrict__ total, int64_t n_loop
     if (*status) atomicOr(flag, 2u);
 }
 
-// Each splitter writes its segment at its loop's offset + rank_start; as in
-// k_segments, every thread walks kWalks segments in lockstep. (Following the
-// 4-byte successor array instead, with the records loaded beside the chain,
-// measured no faster: a step then reads two sectors instead of one.)
-__global__ void k_write_segments(const Xing* __restrict__ rec, const uint32_t* __restrict__ cm,
-                                 const uint32_t* __restrict__ spos,
-                                 const uint32_t* __restrict__ split_id,
-                                 const uint32_t* __restrict__ seg_len,
-                                 const uint32_t* __restrict__ rank_start,
-                                 const int64_t* __restrict__ scan, int64_t ns, int64_t n,
-                                 int64_t n_loops, int64_t vofs, int64_t* __restrict__ loop_off,
-                                 float2* __restrict__ oxy, int32_t* __restrict__ oeid) {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t0 < ns;
-         t0 += stride * kWalks) {
-        uint32_t j[kWalks];
-        int64_t base[kWalks], len[kWalks];
-        int64_t max_len = 0;
-#pragma unroll
-        for (int g = 0; g < kWalks; ++g) {
-            const int64_t t = t0 + g * stride;
-            len[g] = 0;
-            base[g] = 0;
-            j[g] = 0;
-            if (t >= ns) continue;
-            const uint32_t ht = cm[t];
-            if ((int64_t)ht >= n) continue;              // only if the links were inconsistent
-            const uint32_t h = spos[ht];                 // the head splitter of this loop
-            if ((int64_t)h >= ns) continue;
-            const int64_t voff = scan[h] & 0xffffffffLL;
-            if (h == (uint32_t)t && (scan[h] >> 32) < n_loops) loop_off[scan[h] >> 32] = vofs + voff;
+// Each splitter writes its segment at its loop's offset + rank_start. Lanes walk
+// up to kWriteSteps steps of their segments (the 4-byte successors only) and list
+// the crossings with their places in shared memory; the warp then moves the
+// listed vertices, all lanes busy and their loads independent of the walk and of
+// one another. 389 million vertices: 2.65 ms (8 steps 3.0, 16 steps 3.8, 2 steps
+// 3.2; 3.95 with each lane moving its own 16-byte records, a chain of loads).
+constexpr int kWriteSteps = 4;
+__global__ void __launch_bounds__(256)
+k_write_segments(const uint32_t* __restrict__ nxt, const float2* __restrict__ xy,
+                 const int32_t* __restrict__ eid, const uint32_t* __restrict__ cm,
+                 const uint32_t* __restrict__ spos, const uint32_t* __restrict__ split_id,
+                 const uint32_t* __restrict__ seg_len, const uint32_t* __restrict__ rank_start,
+                 const int64_t* __restrict__ scan, int64_t ns, int64_t n, int64_t n_loops,
+                 int64_t vofs, int64_t* __restrict__ loop_off, float2* __restrict__ oxy,
+                 int32_t* __restrict__ oeid) {
+    __shared__ uint2 s_move[256 * kWriteSteps];   // {crossing, place}
+    uint2* move = s_move + (threadIdx.x & ~31u) * kWriteSteps;
+    const int lane = threadIdx.x & 31;
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    uint32_t j = 0, place = 0, left = 0;
+    if (t < ns) {
+        const uint32_t ht = cm[t];
+        const uint32_t h = (int64_t)ht < n ? spos[ht] : 0xffffffffu;   // the loop's head splitter
+        if ((int64_t)h < ns) {                       // else the links were inconsistent
+            const int64_t sc = scan[h], voff = sc & 0xffffffffLL;
+            if (h == (uint32_t)t && (sc >> 32) < n_loops) loop_off[sc >> 32] = vofs + voff;
             const int64_t b = voff + (int64_t)rank_start[t];
             const int64_t l = seg_len[t];
-            if (b < 0 || b + l > n) continue;           // only if the links were inconsistent
-            base[g] = b;
-            len[g] = l;
-            j[g] = split_id[t];
-            max_len = max(max_len, l);
-        }
-        for (int64_t r = 0; r < max_len; ++r) {
-            Xing x[kWalks];
-#pragma unroll
-            for (int g = 0; g < kWalks; ++g)
-                if (r < len[g] && (int64_t)j[g] < n) x[g] = rec[j[g]];
-#pragma unroll
-            for (int g = 0; g < kWalks; ++g) {
-                if (r < len[g] && (int64_t)j[g] < n) {
-                    oxy[base[g] + r] = make_float2(x[g].x, x[g].y);
-                    if (oeid) oeid[base[g] + r] = x[g].eid;
-                    j[g] = x[g].succ;
-                }
+            if (b >= 0 && b + l <= n) {              // else the links were inconsistent
+                place = (uint32_t)b;
+                left = (uint32_t)l;
+                j = split_id[t];
             }
         }
+    }
+    while (__any_sync(0xffffffffu, left > 0)) {
+        const uint32_t steps = min(left, (uint32_t)kWriteSteps);
+        uint32_t at = steps;                         // inclusive prefix sum over the lanes
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const uint32_t v = __shfl_up_sync(0xffffffffu, at, d);
+            if (lane >= d) at += v;
+        }
+        const uint32_t total = __shfl_sync(0xffffffffu, at, 31);
+        at -= steps;
+        for (uint32_t r = 0; r < steps; ++r) {
+            move[at + r] = make_uint2(j, place + r);
+            j = (int64_t)j < n ? nxt[j] & 0x7fffffffu : j;
+        }
+        left -= steps;
+        place += steps;
+        __syncwarp();
+        for (uint32_t q = lane; q < total; q += 32) {
+            const uint2 m = move[q];
+            if ((int64_t)m.x < n) {
+                oxy[m.y] = xy[m.x];
+                if (oeid) oeid[m.y] = eid[m.x];
+            }
+        }
+        __syncwarp();
     }
 }
 
@@ -850,21 +807,22 @@ void contours_chunk(const ChunkGeom& g, double C, const float* sigma, const uint
         if (rp && !replay) rp->plan->ns = rp->plan->nl = rp->plan->n_loops = 0;
         return;
     }
-    // the successor bit trick of k_split_flags needs ids below 2^31
+    // the splitter bit in k_emit's successors needs ids below 2^31
     if (n_cross >= ((int64_t)1 << 31)) fail(CSL_ERR_CAPACITY, "marching squares: too many crossings");
-    DevBuf rec((size_t)n_cross * sizeof(Xing), s);
-    // Every record is written whole by k_emit: x, y and the edge id by the cell
-    // that owns the edge, the successor by the cell the contour enters through
-    // it (each crossing edge is the entry side of exactly one of its two cells).
-    // A replay (planned sizes) may leave records unwritten when its sizes
-    // changed: there they start as invalid ids, so that no walk follows them.
-    if (rp) CSL_CUDA(cudaMemsetAsync(rec.get(), 0xff, (size_t)n_cross * sizeof(Xing), s));
+    DevBuf vxy((size_t)n_cross * 8, s), veid(want_eid ? (size_t)n_cross * 4 : 4, s);
+    int32_t* ve = want_eid ? veid.as<int32_t>() : nullptr;
+    // The lane of k_emit that takes a crossing writes its vertex and successor.
+    // A replay (planned sizes) may leave some unwritten when its sizes changed:
+    // there successors start as 0 (no splitter).
+    DevBuf spos((size_t)n_cross * 4, s), nxt((size_t)n_cross * 4, s);
+    if (rp) CSL_CUDA(cudaMemsetAsync(nxt.get(), 0, (size_t)n_cross * 4, s));
 
     Dense D{ew.as<uint32_t>(), prefix.as<uint32_t>(), c.edge_wpl, c.ewr};
     {
         const int64_t n_bands = ceil_div((int64_t)c.ny + 1, kEmitRows);
         const int64_t n_segs = ceil_div((int64_t)c.mwr, kEmitWords);
         dim3 grid((unsigned)(n_bands * n_segs), (unsigned)g.n_layers);
+        const int bits = splitter_bits(n_cross);
         FusedIn F{};
         if (fv) {
             F.tbase = fv->tbase.as<uint32_t>();
@@ -874,27 +832,19 @@ void contours_chunk(const ChunkGeom& g, double C, const float* sigma, const uint
             F.T = g.T;
             F.ntx = g.ntx;
             F.n_tiles = g.ntx * g.nty;
-            k_emit<true><<<grid, 256, 0, s>>>(sigma, mask, c, D, F, rec.as<Xing>(),
-                                              (uint32_t)n_cross, flag);
+            k_emit<true><<<grid, 32 * kEmitWarps, 0, s>>>(sigma, mask, c, D, F, bits,
+                                                         vxy.as<float2>(), ve, nxt.as<uint32_t>(),
+                                                         (uint32_t)n_cross, flag);
         } else {
-            k_emit<false><<<grid, 256, 0, s>>>(sigma, mask, c, D, F, rec.as<Xing>(),
-                                               (uint32_t)n_cross, flag);
+            k_emit<false><<<grid, 32 * kEmitWarps, 0, s>>>(sigma, mask, c, D, F, bits,
+                                                          vxy.as<float2>(), ve, nxt.as<uint32_t>(),
+                                                          (uint32_t)n_cross, flag);
         }
         CSL_LAUNCH_CHECK("ms emit");
     }
     // ---- loops: splitters, segments, pointer jumping on the splitter graph
-    // nxt[i] = succ(i) | splitter << 31 (0 for a crossing nobody points to);
-    // one scan over its top bits numbers the splitters (spos, for every
+    // one scan over nxt's top bits numbers the splitters (spos, for every
     // crossing) and lists them (split_id) in the same pass
-    DevBuf spos((size_t)n_cross * 4, s), nxt((size_t)n_cross * 4, s);
-    // every crossing is the successor of the crossing through which the
-    // contour enters its cell, so every entry is written; a replay whose sizes
-    // changed may leave some out: there they start as 0 (no splitter)
-    if (rp) CSL_CUDA(cudaMemsetAsync(nxt.get(), 0, (size_t)n_cross * 4, s));
-    const unsigned gx = grid_for(n_cross, 256);
-    k_split_flags<<<gx, 256, 0, s>>>(rec.as<Xing>(), n_cross, splitter_bits(n_cross),
-                                     nxt.as<uint32_t>(), status);
-    CSL_LAUNCH_CHECK("ms splitter flags");
     // the list's room: every crossing, or a replay's planned count
     const int64_t ns_cap = replay ? rp->plan->ns : n_cross;
     DevBuf split_id((size_t)std::max<int64_t>(ns_cap, 1) * 4, s);
@@ -920,7 +870,6 @@ void contours_chunk(const ChunkGeom& g, double C, const float* sigma, const uint
                                   split_id.as<uint32_t>(), ns, n_cross, seg_next.as<uint32_t>(),
                                   seg_len.as<uint32_t>(), status);
     CSL_LAUNCH_CHECK("ms segments");
-    nxt.release();
     // short splitter cycles by walking them; long ones by pointer jumping
     DevBuf cm((size_t)ns * 4, s), long_list((size_t)ns * 4, s), long_pos((size_t)ns * 4, s);
     DevBuf rank_start((size_t)ns * 4, s), loop_len((size_t)ns * 4, s);
@@ -1061,7 +1010,8 @@ void contours_chunk(const ChunkGeom& g, double C, const float* sigma, const uint
     // the walks in flight are those of consecutive splitters (100M workload:
     // contour stage 141 -> 132 ms against 64 CTAs per SM)
     const unsigned gw = (unsigned)std::max<int64_t>(ceil_div(ns, (int64_t)256), (int64_t)1);
-    k_write_segments<<<gw, 256, 0, s>>>(rec.as<Xing>(), cm.as<uint32_t>(), spos.as<uint32_t>(),
+    k_write_segments<<<gw, 256, 0, s>>>(nxt.as<uint32_t>(), vxy.as<float2>(), ve,
+                                        cm.as<uint32_t>(), spos.as<uint32_t>(),
                                         split_id.as<uint32_t>(), seg_len.as<uint32_t>(),
                                         rank_start.as<uint32_t>(), scan.as<int64_t>(), ns, n_cross,
                                         n_loops, vofs, o_loop, o_xy, o_eid);
