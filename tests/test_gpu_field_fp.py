@@ -279,3 +279,28 @@ def test_fused_vertex_lists_grow_when_the_first_guess_is_short():
     b = lat.slice(**g, edge_ids=True, field_kernel="footprint")
     assert a.xy.shape[0] > 2 * 1200 * 1200 // 4   # more than the first guess
     _same_contours(a, b)
+
+
+@pytest.mark.parametrize("R", [0.18, 0.41])
+@pytest.mark.parametrize("uz", [0.05, 0.0999, 0.1001, 0.3, 0.7071, 0.95])
+def test_footprint_rows_of_tilted_struts(uz, R):
+    """Struts of every azimuth at one tilt, on both sides of the one from which the
+    line's ellipse bounds the rows, long ones and ones shorter than the support,
+    against the oracle."""
+    rng = np.random.default_rng(int(1e4 * uz))
+    n = 36
+    phi = 2.0 * np.pi * np.arange(n) / n
+    u = np.stack([np.sqrt(1 - uz * uz) * np.cos(phi), np.sqrt(1 - uz * uz) * np.sin(phi),
+                  np.full(n, uz)], 1)
+    a = rng.uniform([1.0, 1.0, 0.2], [4.0, 4.0, 0.6], (n, 3))
+    length = np.where(np.arange(n) % 3 == 0, 0.15, 1.3)
+    nodes = np.concatenate([a, a + u * length[:, None]]).astype(np.float32)
+    edges = np.stack([np.arange(n), np.arange(n) + n], 1).astype(np.int32)
+    radius = np.full(n, R / 1.5, np.float32)
+    cfg = dict(nodes=nodes, edges=edges, radius=radius, R=R, C=1.0, z0=0.1, dz=0.15,
+               n_layers=8, x0=0.0, y0=0.0, nx=107, ny=103, pixel=0.05)
+    lat = _cs().Lattice(nodes, edges, radius, R=R)
+    sig, cont, g = _slice(lat, cfg, field_kernel="footprint")
+    ref = _oracle(cfg, g)
+    helpers.assert_field(sig, ref, 1.0)
+    assert np.max(ref) > 1.0
