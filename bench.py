@@ -31,19 +31,19 @@ sys.path.insert(0, ROOT)
 
 METRIC = "pixel-evals/s and layers/s at 10M and 100M struts; backward/forward time ratio"
 F_PAIR = 36            # FP32 flops of one (pixel, layer, edge) term in the field kernel
-# Per field kernel, from an ncu capture of one launch on the 12.96M-strut
-# graded lattice (profiles/): the FP32 instructions it executes per cycle as a
-# fraction of the FP32 peak (every evaluated lane), and its DRAM bytes (read +
-# write) per pixel-layer (scaled by pixel-layers to a launch of the timed
-# workload). None where no capture of the current kernel exists.
+# Per field kernel, from an ncu capture of one launch on a 1.6M-strut graded
+# lattice, 1000^2 px x 120 layers (profiles/): the FP32 instructions it executes
+# per cycle as a fraction of the FP32 peak (every evaluated lane), and its DRAM
+# bytes (read + write) per pixel-layer (scaled by pixel-layers to a launch of the
+# timed workload). None where no capture of the current kernel exists.
 NCU_FIELD = {
-    "block": {"kernel": "k_field", "executed_frac": (2 * 2564.8 + 1382.6 + 2056.6) / (152 * 128 * 2),
-              "dram_bytes_per_pixel_layer": (1.212995e9 + 4.259346e9) / (264 * 2000 * 2000),
-              "profile": "profiles/k_field_graded-10M.txt"},
+    "block": {"kernel": "k_field", "executed_frac": (2 * 2543.9 + 1367.4 + 2033.7) / (152 * 128 * 2),
+              "dram_bytes_per_pixel_layer": (0.128309e9 + 0.435139e9) / (120 * 1000 * 1000),
+              "profile": "profiles/field_kernels.txt"},
     "footprint": {"kernel": "k_field_fp",
-                  "executed_frac": (2 * 3131.6 + 1369.7 + 1618.9) / (152 * 128 * 2),
-                  "dram_bytes_per_pixel_layer": (0.729793e9 + 4.292423e9) / (264 * 2000 * 2000),
-                  "profile": "profiles/k_field_fp_graded-10M.txt"},
+                  "executed_frac": (2 * 2973.3 + 1293.7 + 1552.0) / (152 * 128 * 2),
+                  "dram_bytes_per_pixel_layer": (0.078409e9 + 0.438833e9) / (120 * 1000 * 1000),
+                  "profile": "profiles/field_kernels.txt"},
 }
 # The volume fraction's FP32 work beyond the field term: per sample, the
 # sigmoid and the mean (forward), the sigmoid and alpha (the adjoint's pass 1);
@@ -54,13 +54,13 @@ VF_FLOPS_PER_SAMPLE = 4
 VF_GRAD_FLOPS_PER_SAMPLE = 8
 VF_GRAD_FLOPS_PER_TERM = 124
 # Executed FP32 fractions of the volume-fraction kernels from one ncu capture
-# each on the 1M-strut Freudenthal lattice: FFMA (2 flops), FADD and FMUL
+# each on a Freudenthal lattice of 27^3 nodes, 32^3 cells x 8^3 samples: FFMA (2 flops), FADD and FMUL
 # thread instructions per cycle over the FP32 peak per cycle.
 NCU_VF = {"forward": {"kernel": "k_field",
-                      "executed_frac": (2 * 4094.3 + 1978.2 + 3107.9) / (152 * 128 * 2)},
+                      "executed_frac": (2 * 4031.1 + 1949.8 + 3057.9) / (152 * 128 * 2)},
           "backward": {"kernel": "k_vf_grad",
-                       "executed_frac": (2 * 2256.0 + 1117.7 + 2062.3) / (152 * 128 * 2)},
-          "profile": "profiles/k_vf_grad_freudenthal-1M.txt"}
+                       "executed_frac": (2 * 341.7 + 620.1 + 314.7) / (152 * 128 * 2)},
+          "profile": "profiles/other_kernels.txt"}
 HBM_GBS = 6772.9       # measured copy bandwidth of the GPU
 # algorithmic bytes of the HBM-bound stages
 BIN_BYTES_PER_WINDOW_RECORD = 24   # xy box (16) + z range (8) of a record read per slab window
@@ -801,7 +801,7 @@ def main():
             "frac": achieved / peak,
             "traffic": (ncu["dram_bytes_per_pixel_layer"] * px_layers_per_launch
                         if ncu["dram_bytes_per_pixel_layer"] else None),
-            "traffic_basis": "ncu dram bytes of one field launch on the 12.96M-strut graded "
+            "traffic_basis": "ncu dram bytes of one field launch on a 1.6M-strut graded "
                              "lattice, scaled by pixel-layers per launch",
             "kernel": ncu["kernel"], "flops_per_term": F_PAIR,
             "nonzero_terms_per_step": pairs, "evaluated_terms_per_step": evaluated,
@@ -817,7 +817,7 @@ def main():
     roof["peak_check_ffma_microbenchmark_tflops"] = ffma_tflops
     roof["executed_frac_ncu"] = ncu["executed_frac"]
     roof["executed_basis"] = ("ncu FFMA + FADD + FMUL thread instructions per cycle of one "
-                              "field launch on the 12.96M-strut graded lattice, every evaluated "
+                              "field launch on a 1.6M-strut graded lattice, every evaluated "
                               f"lane included ({ncu['profile']})")
     # the HBM-bound stages, against the measured copy bandwidth: algorithmic
     # bytes (the minimum each stage must move) over its event-timed duration

@@ -12,8 +12,8 @@
 //   2. a prefix sum of the edge words' popcounts numbers the crossings in
 //      (layer, edge id) order: id = prefix[word] + popc(lower bits);
 //   3. k_emit: per crossing, its vertex (the zero of the linear interpolant of
-//      Sigma - C) and the crossings before and after it, each the other
-//      crossing side of one of the two cells that share the edge. Walking a
+//      Sigma - C) and its successor, the other crossing side of the one of the
+//      two cells sharing the edge that the contour enters there. Walking a
 //      cell's sides counter-clockwise, a side from an inside to an outside
 //      corner is an entry, from outside to inside an exit; a saddle (two
 //      inside corners on a diagonal) joins its inside corners when the mean of
@@ -24,8 +24,9 @@
 //      of crossings; each splitter walks its segment to the next
 //      splitter, so no thread walks a whole long loop;
 //   5. on the graph of splitters (one cycle per loop), a cycle of at most 16
-//      splitters (every small loop) is resolved by walking it; on the rest,
-//      pointer jumping gives every splitter its cycle's minimum (the head)
+//      splitters (32 in small chunks; every small loop) is resolved by walking
+//      it; on the rest, pointer jumping (by one block in shared memory up to
+//      kLongBlock splitters, by the grid above) gives every splitter its cycle's minimum (the head)
 //      and, with the cycles cut before their heads, weighted list ranking
 //      gives every segment its distance from the head;
 //   6. a prefix sum over the heads (loop length) numbers the loops in head
@@ -123,12 +124,12 @@ __device__ __forceinline__ float2 fused_vertex(const FusedIn& F, const Dense& D,
     return F.verts[(int64_t)F.tbase[tl] + F.roff[tl * (F.T + 1) + b + 1] + rank];
 }
 
-
 // A block of k_emit covers a band of kEmitRows sample rows and kEmitWords mask
 // words (32 samples each) of one layer, a warp per row at a time. A lane takes a
 // crossing: it computes the vertex and, from the two cells that share the
-// edge, the crossings before and after it on the contour, so that records and
-// successors are written whole and in order, and the splitters are known here.
+// edge, the crossing after it on the contour and whether it is a local minimum,
+// so that vertices and successors are written in order and the splitters are
+// known here.
 // The crossings of a warp's row are listed in shared memory first (ids are
 // consecutive along a row), which keeps every lane busy; edge words and their
 // prefix sums of the band and of one row and one word around it are staged as
