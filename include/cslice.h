@@ -325,8 +325,8 @@ typedef struct csl_cells {
  * the density of Eq. 9 with the Monte-Carlo hit count replaced by stratified
  * samples and a sigmoid, so that it is differentiable (radius tuning, Sec.
  * 5.4). vf_out: device float[dims[2]][dims[1]][dims[0]] (caller-owned).
- * Errors: INVALID_ARG for bad cells (see csl_cells) or NULL pointers.
- * Synchronises the stream.
+ * Errors: INVALID_ARG for bad cells (see csl_cells) or NULL pointers, TIMEOUT
+ * when a bounded wait of the field kernel gave up. Synchronises the stream.
  */
 csl_status csl_volume_fraction(csl_lattice* lat, const csl_cells* cells, float* vf_out,
                                void* stream);
@@ -344,7 +344,8 @@ csl_status csl_volume_fraction(csl_lattice* lat, const csl_cells* cells, float* 
  *   grad_radius  device float[n_edges]   (overwritten)
  *   grad_nodes   device float[n_nodes][3] (overwritten)
  * The sums run in a fixed order: results are deterministic.
- * Synchronises the stream.
+ * Errors: as csl_volume_fraction; TIMEOUT when a bounded wait of the field
+ * kernel gave up (the gradients are then unspecified). Synchronises the stream.
  */
 csl_status csl_volume_fraction_backward(csl_lattice* lat, const csl_cells* cells,
                                         const float* grad_vf, float* grad_radius,
@@ -544,6 +545,15 @@ csl_status csl_support_metrics(const csl_lattice* lat, const double* t_p, double
  * the device stays usable. The paper has no counterpart.
  */
 csl_status csl_debug_wait_timeout(uint32_t polls, void* stream);
+
+/*
+ * csl_debug_lattice_timeout -- the same wait reporting where the field kernel
+ * reports: it gives up after `polls` polls (1 .. 2^22) and sets the lattice's
+ * status word, so that the next call that evaluates the field of lat returns
+ * CSL_ERR_TIMEOUT (and clears the word). For tests of those calls. The paper
+ * has no counterpart. Synchronises the stream.
+ */
+csl_status csl_debug_lattice_timeout(csl_lattice* lat, uint32_t polls, void* stream);
 
 /*
  * csl_measure_fp32_peak -- FP32 throughput of the device, measured with a

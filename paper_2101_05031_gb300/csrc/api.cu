@@ -1062,6 +1062,8 @@ csl_status csl_volume_fraction_backward(csl_lattice* L, const csl_cells* cells,
         launches_and_reset();
         vf_backward(L, *cells, grad_vf, grad_radius, grad_nodes, s);
         CSL_CUDA(cudaStreamSynchronize(s));
+        // Sigma is recomputed by the field kernel, whose bulk copies may give up
+        check_lattice_status(L, s);
         t_stats = csl_stats{};
         t_stats.kernel_launches = launches_and_reset();
     });

@@ -578,17 +578,23 @@ void field_batch_run(FieldBatch& fb, int n_ctas, cudaStream_t s) {
 
 }  // namespace csl
 
-extern "C" csl_status csl_debug_wait_timeout(uint32_t polls, void* stream) {
+namespace {
+
+csl_status wait_nothing(uint32_t polls, cudaStream_t s, uint32_t* err, bool report) {
     try {
         if (polls == 0 || polls > csl::kWaitLimit) csl::fail(CSL_ERR_INVALID_ARG, "polls in [1, 2^22]");
-        cudaStream_t s = (cudaStream_t)stream;
-        csl::DevBuf err(4, s);
-        CSL_CUDA(cudaMemsetAsync(err.get(), 0, 4, s));
-        csl::k_wait_nothing<<<1, 64, 0, s>>>(polls, err.as<uint32_t>());
+        csl::DevBuf own;
+        if (!err) {
+            own.alloc(4, s);
+            err = own.as<uint32_t>();
+            CSL_CUDA(cudaMemsetAsync(err, 0, 4, s));
+        }
+        csl::k_wait_nothing<<<1, 64, 0, s>>>(polls, err);
         CSL_LAUNCH_CHECK("wait test");
         uint32_t st = 0;
-        csl::read_to_host(&st, err.get(), 4, s);
-        if (st & csl::ST_TIMEOUT) csl::fail(CSL_ERR_TIMEOUT, "the wait gave up as it should");
+        csl::read_to_host(&st, err, 4, s);
+        if (report && (st & csl::ST_TIMEOUT))
+            csl::fail(CSL_ERR_TIMEOUT, "the wait gave up as it should");
         return CSL_OK;
     } catch (const csl::Error& e) {
         csl::set_last_error(e.what());
@@ -597,4 +603,18 @@ extern "C" csl_status csl_debug_wait_timeout(uint32_t polls, void* stream) {
         csl::set_last_error("unknown error");
         return CSL_ERR_CUDA;
     }
+}
+
+}  // namespace
+
+extern "C" csl_status csl_debug_wait_timeout(uint32_t polls, void* stream) {
+    return wait_nothing(polls, (cudaStream_t)stream, nullptr, true);
+}
+
+extern "C" csl_status csl_debug_lattice_timeout(csl_lattice* L, uint32_t polls, void* stream) {
+    if (!L) {
+        csl::set_last_error("lattice is NULL");
+        return CSL_ERR_INVALID_ARG;
+    }
+    return wait_nothing(polls, (cudaStream_t)stream, L->status.as<uint32_t>(), false);
 }
