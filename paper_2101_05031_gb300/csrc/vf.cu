@@ -271,6 +271,9 @@ k_vf_grad(const csl_rec* __restrict__ recs, const uint32_t* __restrict__ tstart,
             const float ex = fmaf(-t0, ux, dx), ey = fmaf(-t0, uy, dy);
             const float ez = fmaf(-t0, uz, dz);
             const float h2 = fmaxf(c.R2 - fmaf(ez, ez, fmaf(ey, ey, ex * ex)), 0.0f);
+            // out of reach (the rows are widened, the columns of an edge along x are its
+            // box): no term, also where alpha is infinite or NaN
+            if (h2 == 0.0f) continue;
             const float w = sqrt_approx(h2);
             const float tau1 = fmaxf(-t0, -w), tau2 = fminf(len - t0, w);
             const float hh = 0.5f * fmaxf(tau2 - tau1, 0.0f);   // half width
