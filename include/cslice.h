@@ -33,7 +33,14 @@
  * allocator (cudaMallocAsync) on that stream and frees it the same way; what
  * outlives the call (a lattice, a batch) comes from the same pool on the
  * legacy default stream, synchronised, and is freed after a device
- * synchronisation. Freed memory stays in the pool for later calls.
+ * synchronisation. Freed memory stays in the pool for later calls. Device
+ * arrays of results other than those of csl_slice_layers (contours of batches,
+ * simplified or uploaded contours, infill) of up to 256 MiB come from the pool
+ * too, while those not yet freed stay below 1 GiB together (larger ones, and
+ * more of them, from cudaMalloc): memory of the pool has no legacy IPC handles
+ * and needs a pool access setting for peer access. The result's free call
+ * returns such an array to the pool, after waiting for the device that holds
+ * it, whichever device is current.
  */
 #ifndef CSLICE_H
 #define CSLICE_H

@@ -124,14 +124,21 @@ size_t vertex_block_eid_offset(size_t block_bytes, bool want_eid);
 csl_contours* new_host_contours(int32_t n_layers, int64_t n_loops, int64_t n_verts, bool want_eid,
                                 void* vertex_block = nullptr);
 
-// Device memory for arrays handed to the caller (contours, infill). Up to
-// kResultPoolBytes from the stream-ordered pool, where the next result finds it
-// again (a cudaMalloc and cudaFree of such arrays take 40 to 100 us each: for
-// the contours of 12 batched lattices 2.6 ms beside 9.7 ms of kernels), larger
-// ones from cudaMalloc so that the pool keeps none of them. Ordered on s: the
-// caller synchronises s before the array is handed out. CSL_ERR_OOM with `what`
-// when there is none. result_free waits for the device, as cudaFree does.
+// Keep freed workspace in the current device's stream-ordered pool.
+void keep_pool_memory();
+
+// Device memory for arrays handed to the caller (contours, infill; results.cu).
+// Arrays of up to kResultPoolBytes come from the stream-ordered pool, where the
+// next result or workspace finds them again (a cudaMalloc and cudaFree of such
+// arrays take 40 to 100 us each: for the contours of 12 batched lattices 2.6 ms
+// beside 9.7 ms of kernels), while those in the caller's hands stay below
+// kResultPoolTotal together, which bounds what results can leave in the pool;
+// others come from cudaMalloc. Ordered on s: the caller synchronises s before
+// the array is handed out. CSL_ERR_OOM with `what` when there is none.
+// result_free waits for the device that holds the array, whichever is current,
+// as cudaFree does.
 constexpr size_t kResultPoolBytes = (size_t)256 << 20;
+constexpr size_t kResultPoolTotal = (size_t)1 << 30;
 void* result_alloc(size_t bytes, cudaStream_t s, const char* what);
 void result_free(void* p);
 

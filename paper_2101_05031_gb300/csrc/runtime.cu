@@ -6,7 +6,6 @@
 #include <mutex>
 #include <new>
 #include <unordered_map>
-#include <unordered_set>
 #include <utility>
 #include <vector>
 
@@ -73,7 +72,7 @@ int64_t device_bytes_peak() { return g_peak.load(); }
 
 // Keep freed workspace in the stream-ordered pool instead of returning it to
 // the CUDA driver at every synchronisation (per process, per device).
-static void keep_pool_memory() {
+void keep_pool_memory() {
     static thread_local int done_for = -1;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev == done_for) return;
@@ -213,45 +212,6 @@ void* host_block_take_largest(size_t* bytes) {
     g_host_free_bytes -= it->first;
     g_host_free.erase(it);
     return p;
-}
-
-namespace {
-std::mutex g_result_mu;
-std::unordered_set<void*> g_result_pooled;   // result arrays that came from the pool
-}  // namespace
-
-void* result_alloc(size_t bytes, cudaStream_t s, const char* what) {
-    if (bytes == 0) bytes = 16;
-    void* p = nullptr;
-    if (bytes <= kResultPoolBytes) {
-        keep_pool_memory();
-        if (cudaMallocAsync(&p, bytes, s) == cudaSuccess) {
-            std::lock_guard<std::mutex> lk(g_result_mu);
-            g_result_pooled.insert(p);
-            return p;
-        }
-        cudaGetLastError();
-    }
-    if (cudaMalloc(&p, bytes) != cudaSuccess) {
-        cudaGetLastError();
-        fail(CSL_ERR_OOM, what);
-    }
-    return p;
-}
-
-void result_free(void* p) {
-    if (!p) return;
-    bool pooled = false;
-    {
-        std::lock_guard<std::mutex> lk(g_result_mu);
-        pooled = g_result_pooled.erase(p) > 0;
-    }
-    if (!pooled) {
-        cudaFree(p);
-        return;
-    }
-    cudaDeviceSynchronize();   // any stream may still use it
-    cudaFreeAsync(p, 0);
 }
 
 size_t vertex_block_eid_offset(size_t block_bytes, bool want_eid) {
