@@ -296,7 +296,7 @@ extern "C" csl_status csl_render_depth(const csl_lattice* L, const csl_camera* c
         c.half_w = (float)(tan(0.5 * cam->fov_y) * cam->width / cam->height);
         c.width = cam->width;
         c.height = cam->height;
-        c.tiles_x = (cam->width + 15) / 16;
+        c.tiles_x = (cam->width - 1) / 16 + 1;   // up to 2^31 - 1 pixels
         c.step = (float)cam->step;
         c.refine = cam->refine;
         for (int k = 0; k < 3; ++k) {
@@ -385,7 +385,7 @@ extern "C" csl_status csl_render_depth(const csl_lattice* L, const csl_camera* c
         k_rv_bounds<<<grid_for(n_pairs, 256), 256, 0, s>>>(d_k.as<uint32_t>(), n_pairs,
                                                            d_cb.as<uint32_t>(), d_ce.as<uint32_t>());
         CSL_LAUNCH_CHECK("render cell bounds");
-        const int64_t n_blocks = (int64_t)c.tiles_x * ((cam->height + 7) / 8);
+        const int64_t n_blocks = (int64_t)c.tiles_x * ((cam->height - 1) / 8 + 1);
         k_rv_render<<<(unsigned)n_blocks, 128, 0, s>>>(rec, d_v.as<uint32_t>(), d_cb.as<uint32_t>(),
                                                        d_ce.as<uint32_t>(), g, c, depth);
         CSL_LAUNCH_CHECK("render rays");
