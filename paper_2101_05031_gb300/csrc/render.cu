@@ -26,6 +26,7 @@ namespace {
 struct RvGrid {
     float lox, loy, loz, h, inv_h;   // grid corner and cell edge
     float reach;   // R plus a slack far above the rounding of a sample's position and cell
+    float near;    // reach plus that slack again, for the ranges of cells along a strut
     int32_t nx, ny, nz;
 };
 
@@ -43,10 +44,26 @@ struct RvConst {
     float R2, inv_R4, C;
 };
 
+// Narrows [t0, t1] to the part of a strut whose coordinate s + t u lies in
+// [lo, hi] (inv = 1 / u, 0 where the strut runs across the axis).
+__device__ __forceinline__ void clip_strut(float lo, float hi, float s, float inv, float& t0,
+                                           float& t1) {
+    if (inv == 0.0f) return;
+    const float a = (lo - s) * inv, b = (hi - s) * inv;
+    t0 = fmaxf(t0, fminf(a, b));
+    t1 = fminf(t1, fmaxf(a, b));
+}
+
 // Calls f(cell) for every cell that the strut's support (radius R with its
 // slack) can meet: the cells of its box, without those that the strut's line
 // passes farther than R from (the separating axis from the line to the
-// centre; a cell reaches at most h/2 |e|_1 / |e| along it).
+// centre; a cell reaches at most h/2 |e|_1 / |e| along it). Of a layer of cells
+// only the rows beside the part of the strut that comes near the layer are
+// looked at, of a row only the cells beside the part that comes near the row, so
+// that a strut costs as many tests as it lists cells, about: a depth image of one
+// strut of 140 mm, R = 0.5 mm, across its box takes 1.7 ms, 203 ms with the whole
+// box tested by the strut's thread, of 500 of them 2.8 and 332 ms (429,039 struts of
+// about 1 mm: the same 4.1 ms either way).
 template <class F>
 __device__ __forceinline__ void strut_cells(const csl_rec& r, const RvGrid& g, F f) {
     const float R = g.reach;
@@ -60,11 +77,26 @@ __device__ __forceinline__ void strut_cells(const csl_rec& r, const RvGrid& g, F
         a[k] = max(0, min(n[k] - 1, (int)floorf((lo - o[k]) * g.inv_h)));
         b[k] = max(0, min(n[k] - 1, (int)floorf((hi - o[k]) * g.inv_h)));
     }
+    const float W = g.near;
+    const float inv_y = fabsf(r.uy) > 1e-12f ? 1.0f / r.uy : 0.0f;
+    const float inv_z = fabsf(r.uz) > 1e-12f ? 1.0f / r.uz : 0.0f;
     for (int k = a[2]; k <= b[2]; ++k) {
-        const float qz = g.loz + g.h * ((float)k + 0.5f) - r.az;
-        for (int j = a[1]; j <= b[1]; ++j) {
-            const float qy = g.loy + g.h * ((float)j + 0.5f) - r.ay;
-            for (int i = a[0]; i <= b[0]; ++i) {
+        const float z = g.loz + g.h * (float)k, qz = g.loz + g.h * ((float)k + 0.5f) - r.az;
+        float t0 = 0.0f, t1 = r.len;
+        clip_strut(z - W, z + g.h + W, r.az, inv_z, t0, t1);
+        if (t0 > t1) continue;
+        const float ya = r.ay + t0 * r.uy, yb = r.ay + t1 * r.uy;
+        const int j0 = max(a[1], (int)floorf((fminf(ya, yb) - W - g.loy) * g.inv_h));
+        const int j1 = min(b[1], (int)floorf((fmaxf(ya, yb) + W - g.loy) * g.inv_h));
+        for (int j = j0; j <= j1; ++j) {
+            const float y = g.loy + g.h * (float)j, qy = g.loy + g.h * ((float)j + 0.5f) - r.ay;
+            float s0 = t0, s1 = t1;
+            clip_strut(y - W, y + g.h + W, r.ay, inv_y, s0, s1);
+            if (s0 > s1) continue;
+            const float xa = r.ax + s0 * r.ux, xb = r.ax + s1 * r.ux;
+            const int i0 = max(a[0], (int)floorf((fminf(xa, xb) - W - g.lox) * g.inv_h));
+            const int i1 = min(b[0], (int)floorf((fmaxf(xa, xb) + W - g.lox) * g.inv_h));
+            for (int i = i0; i <= i1; ++i) {
                 const float qx = g.lox + g.h * ((float)i + 0.5f) - r.ax;
                 const float t = qx * r.ux + qy * r.uy + qz * r.uz;
                 const float ex = qx - t * r.ux, ey = qy - t * r.uy, ez = qz - t * r.uz;
@@ -354,6 +386,7 @@ extern "C" csl_status csl_render_depth(const csl_lattice* L, const csl_camera* c
         for (int k = 0; k < 3; ++k)
             scale = std::max({scale, fabs((double)c.blo[k]), fabs((double)c.bhi[k])});
         g.reach = (float)(R + 1e-3 * R + 4e-6 * scale);
+        g.near = (float)(R + 1e-3 * R + 8e-6 * scale);
         const csl_rec* rec = L->rec.as<csl_rec>();
         DevBuf d_cnt((size_t)ne * 4, s), d_off((size_t)ne * 8, s), d_tot(8, s);
         int64_t n_cells = 0, n_pairs = 0;
