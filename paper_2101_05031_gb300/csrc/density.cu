@@ -255,52 +255,65 @@ struct TetBox {
 // interpolated target at the centroid. A lane per tetrahedron while it has
 // few candidate centres (FP64 set-up that is the same in every lane of a warp
 // costs as much for one tetrahedron as for 32: with a warp per tetrahedron 451,000
-// of them took 6.7 ms, now 0.29 ms); the warp shares the candidates of the
-// others.
+// of them took 6.7 ms, now 0.29 ms). The others are listed for
+// k_dm_target_many, a warp each: taken one after another by the warp that met
+// them, 48 tetrahedra with some 64,000 candidates each kept two warps of the chip
+// busy for 191 ms; 8.1 ms so.
 constexpr int kDmOwn = 16;
+
+__device__ __forceinline__ void dm_store_target(const TetBox& b, const GridConst& g,
+                                                const float* __restrict__ tgt, double best,
+                                                bool found, double* __restrict__ out) {
+    const double3 c = make_double3((b.v[0].x + b.v[1].x + b.v[2].x + b.v[3].x) * 0.25,
+                                   (b.v[0].y + b.v[1].y + b.v[2].y + b.v[3].y) * 0.25,
+                                   (b.v[0].z + b.v[1].z + b.v[2].z + b.v[3].z) * 0.25);
+    *out = found ? best : trilinear(g, tgt, c);
+}
+
 __global__ void k_dm_target(const float4* __restrict__ tv, int64_t n_tets, GridConst g,
-                            const float* __restrict__ tgt, double* __restrict__ out) {
-    const int lane = threadIdx.x & 31;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t t0 = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31u); t0 < n_tets;
-         t0 += stride) {
-        const int64_t t = t0 + lane;
+                            const float* __restrict__ tgt, double* __restrict__ out,
+                            uint32_t* __restrict__ many, uint32_t* __restrict__ n_many) {
+    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n_tets;
+         t += (int64_t)gridDim.x * blockDim.x) {
+        TetBox b;
+        b.load(tv + 4 * t, g);
+        if (b.cnt > kDmOwn) {
+            // one addition for the lanes that are here together (any grouping of them is
+            // right: the list's order does not matter)
+            const uint32_t act = __activemask(), lane = threadIdx.x & 31;
+            uint32_t at = 0;
+            if (lane == __ffs(act) - 1u) at = atomicAdd(n_many, (uint32_t)__popc(act));
+            at = __shfl_sync(act, at, __ffs(act) - 1);
+            many[at + __popc(act & ((1u << lane) - 1u))] = (uint32_t)t;
+            continue;
+        }
         double best = -INFINITY;
         bool found = false;
-        int64_t cnt = 0;
-        double3 c = make_double3(0.0, 0.0, 0.0);
-        if (t < n_tets) {
-            TetBox b;
-            b.load(tv + 4 * t, g);
-            c = make_double3((b.v[0].x + b.v[1].x + b.v[2].x + b.v[3].x) * 0.25,
-                             (b.v[0].y + b.v[1].y + b.v[2].y + b.v[3].y) * 0.25,
-                             (b.v[0].z + b.v[1].z + b.v[2].z + b.v[3].z) * 0.25);
-            cnt = b.cnt;
-            if (cnt <= kDmOwn)
-                for (int q = 0; q < (int)cnt; ++q)
-                    b.take(b.i0 + q % b.ni, b.j0 + q / b.ni % b.nj, b.k0 + q / (b.ni * b.nj), g,
-                           tgt, best, found);
-        }
-        uint32_t many = __ballot_sync(0xffffffffu, cnt > kDmOwn);
-        while (many) {
-            const int src = __ffs(many) - 1;
-            many &= many - 1u;
-            TetBox b;
-            b.load(tv + 4 * (t0 + src), g);
-            double m = -INFINITY;
-            bool f = false;
-            for (int64_t q = lane; q < b.cnt; q += 32)
-                b.take(b.i0 + (int)(q % b.ni), b.j0 + (int)(q / b.ni % b.nj),
-                       b.k0 + (int)(q / ((int64_t)b.ni * b.nj)), g, tgt, m, f);
+        for (int q = 0; q < (int)b.cnt; ++q)
+            b.take(b.i0 + q % b.ni, b.j0 + q / b.ni % b.nj, b.k0 + q / (b.ni * b.nj), g, tgt, best,
+                   found);
+        dm_store_target(b, g, tgt, best, found, out + t);
+    }
+}
+
+__global__ void k_dm_target_many(const float4* __restrict__ tv, const uint32_t* __restrict__ many,
+                                 const uint32_t* __restrict__ n_many, GridConst g,
+                                 const float* __restrict__ tgt, double* __restrict__ out) {
+    const int lane = threadIdx.x & 31;
+    const uint32_t n = *n_many, warps = gridDim.x * (blockDim.x >> 5);
+    for (uint32_t i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < n; i += warps) {
+        const uint32_t t = many[i];
+        TetBox b;
+        b.load(tv + 4 * (int64_t)t, g);
+        double best = -INFINITY;
+        bool found = false;
+        for (int64_t q = lane; q < b.cnt; q += 32)
+            b.take(b.i0 + (int)(q % b.ni), b.j0 + (int)(q / b.ni % b.nj),
+                   b.k0 + (int)(q / ((int64_t)b.ni * b.nj)), g, tgt, best, found);
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
-            f = __any_sync(0xffffffffu, f);
-            if (lane == src) {
-                best = m;
-                found = f;
-            }
-        }
-        if (t < n_tets) out[t] = found ? best : trilinear(g, tgt, c);
+        for (int o = 16; o > 0; o >>= 1) best = fmax(best, __shfl_xor_sync(0xffffffffu, best, o));
+        found = __any_sync(0xffffffffu, found);
+        if (lane == 0) dm_store_target(b, g, tgt, best, found, out + t);
     }
 }
 
@@ -711,7 +724,7 @@ extern "C" csl_status csl_density_match(const float* nodes, int64_t n_nodes, con
         // the level's tetrahedra (the input, then the children of the last
         // level's splits: a contiguous range of ids), then the subdivision.
         // Values are kept per tetrahedron id.
-        DevBuf d_target, d_rho, d_ratio, d_tv, d_split;
+        DevBuf d_target, d_rho, d_ratio, d_tv, d_split, d_many;
         auto per_tet = [&](int64_t used, int64_t need) {
             auto keep = [&](DevBuf& b, size_t el) {
                 if ((size_t)need * el <= b.size()) return;
@@ -733,9 +746,17 @@ extern "C" csl_status csl_density_match(const float* nodes, int64_t n_nodes, con
             double* tgt_d = d_target.as<double>() + t0;
             float* rho_d = d_rho.as<float>() + t0;
             float* rat_d = d_ratio.as<float>() + t0;
+            // those with many candidates (all of them may be), behind their count
+            d_many.ensure((size_t)(nc + 1) * 4, s);
+            uint32_t* n_many = d_many.as<uint32_t>();
+            CSL_CUDA(cudaMemsetAsync(n_many, 0, 4, s));
             k_dm_target<<<grid_for(nc, 128), 128, 0, s>>>(d_tv.as<float4>(), nc, g,
-                                                               d_tgt.as<float>(), tgt_d);
+                                                          d_tgt.as<float>(), tgt_d, n_many + 1,
+                                                          n_many);
             CSL_LAUNCH_CHECK("density targets");
+            k_dm_target_many<<<grid_for(nc * 32, 128), 128, 0, s>>>(
+                d_tv.as<float4>(), n_many + 1, n_many, g, d_tgt.as<float>(), tgt_d);
+            CSL_LAUNCH_CHECK("density targets of large tetrahedra");
             k_dm_tet<<<grid_for(nc * 32, tet_threads), tet_threads, tet_smem, s>>>(
                 d_tv.as<float4>(), tgt_d, nc, d_coef.as<float4>(), n_samples, c, rho_d, rat_d);
             CSL_LAUNCH_CHECK("tetrahedron densities");
