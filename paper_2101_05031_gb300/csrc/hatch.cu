@@ -15,9 +15,10 @@
 // layer * n_lines + m): crossings counted per line, the counts scanned, the x
 // placed in their line's bucket, and a warp per line that sorts its bucket and
 // writes its segments. The order inside a line is that of the x alone (equal x
-// are the same bits), so the slots that atomics hand out do not show. Lines of
-// more than kLineMost crossings, and more lines than vertices (where the lines'
-// counts cost more than the crossings), take radix sorts by x and then by key.
+// are the same bits), so the slots that atomics hand out do not show. Where a line
+// has more than kLineMost crossings the buckets go to radix sorts by x and then by
+// key; so do, without buckets, more lines than vertices (where the lines' counts
+// cost more than the crossings) and few lines for many vertices (kLineVerts).
 #include <math.h>
 #include <string.h>
 
@@ -131,24 +132,63 @@ __device__ __forceinline__ float float_of(uint32_t k) {
     return __uint_as_float((k & 0x80000000u) ? k & 0x7fffffffu : ~k);
 }
 
-// Every crossing of the edge from vertex v: f(key, m).
+// Every crossing of every edge, by whole warps: f(key, m, a, b, peers), peers = the
+// lanes that are at a crossing of the same line now. Contours list their loops row
+// by row, so the lanes of a warp meet the same few lines: an atomic for each group
+// of them instead of one per crossing takes 0.10 ms instead of 1.25 for the counts
+// of 3000 x 1000 squares (12 million crossings on 2,000 lines), which one address
+// after another had held up. Edges of more than kWideEdge lines are taken by all
+// lanes together.
+constexpr int kWideEdge = 32;
 template <class F>
 __device__ __forceinline__ void each_crossing(const float2* __restrict__ xy,
                                               const int64_t* __restrict__ loop_off,
                                               const uint32_t* __restrict__ loop_of,
                                               const uint32_t* __restrict__ layer_of,
-                                              const HatchConst& c, int64_t v, F f) {
-    const uint32_t L = loop_of[v];
-    const int64_t w = v + 1 < loop_off[L + 1] ? v + 1 : loop_off[L];
-    const float2 a = xy[v], b = xy[w];
-    const float lo = fminf(a.y, b.y), hi = fmaxf(a.y, b.y);
-    if (!(lo < hi)) return;
-    const int m0 = first_line_at_or_above(c.ys, c.y0f, c.inv_sp, c.n_lines, lo);
-    int m1 = m0;
-    while (m1 < c.n_lines && c.ys[m1] < hi) ++m1;
-    if (m0 == m1) return;
-    const uint32_t base = layer_of[L] * (uint32_t)c.n_lines;
-    for (int m = m0; m < m1; ++m) f(base + (uint32_t)m, m, a, b);
+                                              const HatchConst& c, F f) {
+    const int lane = threadIdx.x & 31;
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t v0 = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31u); v0 < c.n_verts;
+         v0 += stride) {
+        const int64_t v = v0 + lane;
+        float2 a = make_float2(0.0f, 0.0f), b = a;
+        int m = 0, m1 = 0;
+        uint32_t base = 0;
+        if (v < c.n_verts) {
+            int64_t w;
+            edge_of(loop_off, loop_of, v, w);
+            a = xy[v];
+            b = xy[w];
+            const float lo = fminf(a.y, b.y), hi = fmaxf(a.y, b.y);
+            if (lo < hi) {
+                m = first_line_at_or_above(c.ys, c.y0f, c.inv_sp, c.n_lines, lo);
+                m1 = first_line_at_or_above(c.ys, c.y0f, c.inv_sp, c.n_lines, hi);
+                base = layer_of[loop_of[v]] * (uint32_t)c.n_lines;
+            }
+        }
+        uint32_t wide = __ballot_sync(0xffffffffu, m1 - m > kWideEdge);
+        for (; wide; wide &= wide - 1u) {
+            const int src = __ffs(wide) - 1;
+            const float2 p = make_float2(__shfl_sync(0xffffffffu, a.x, src),
+                                         __shfl_sync(0xffffffffu, a.y, src));
+            const float2 q = make_float2(__shfl_sync(0xffffffffu, b.x, src),
+                                         __shfl_sync(0xffffffffu, b.y, src));
+            const uint32_t pb = __shfl_sync(0xffffffffu, base, src);
+            const int from = __shfl_sync(0xffffffffu, m, src), to = __shfl_sync(0xffffffffu, m1, src);
+            for (int64_t k = from + lane; k < to; k += 32)
+                f(pb + (uint32_t)k, (int)k, p, q, 1u << lane);
+            if (lane == src) m = m1;
+            __syncwarp();
+        }
+        while (const uint32_t act = __ballot_sync(0xffffffffu, m < m1)) {
+            if (m < m1) {
+                const uint32_t key = base + (uint32_t)m;
+                f(key, m, a, b, __match_any_sync(act, key));
+                ++m;
+            }
+            __syncwarp();
+        }
+    }
 }
 
 // Crossings per line.
@@ -156,10 +196,11 @@ __global__ void k_line_count(const float2* __restrict__ xy, const int64_t* __res
                              const uint32_t* __restrict__ loop_of,
                              const uint32_t* __restrict__ layer_of, HatchConst c,
                              uint32_t* __restrict__ hist) {
-    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < c.n_verts;
-         v += (int64_t)gridDim.x * blockDim.x)
-        each_crossing(xy, loop_off, loop_of, layer_of, c, v,
-                      [&](uint32_t key, int, float2, float2) { atomicAdd(hist + key, 1u); });
+    const uint32_t lane = threadIdx.x & 31;
+    each_crossing(xy, loop_off, loop_of, layer_of, c,
+                  [&](uint32_t key, int, float2, float2, uint32_t peers) {
+                      if (lane == __ffs(peers) - 1u) atomicAdd(hist + key, (uint32_t)__popc(peers));
+                  });
 }
 
 // most[0] = the longest line's crossings; a line with an odd count is reported.
@@ -180,29 +221,44 @@ __global__ void k_line_most(const uint32_t* __restrict__ hist, int64_t n_keys,
 }
 
 // Each crossing's x into its line's bucket: the slots left are counted down in
-// hist, which ends at 0.
+// hist, which ends at 0. With keys (lines too long for a warp) the crossings' lines
+// beside them, and x as it is.
 __global__ void k_line_emit(const float2* __restrict__ xy, const int64_t* __restrict__ loop_off,
                             const uint32_t* __restrict__ loop_of,
                             const uint32_t* __restrict__ layer_of, HatchConst c,
                             const int64_t* __restrict__ start, uint32_t* __restrict__ hist,
-                            uint32_t* __restrict__ xs) {
-    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < c.n_verts;
-         v += (int64_t)gridDim.x * blockDim.x)
-        each_crossing(xy, loop_off, loop_of, layer_of, c, v,
-                      [&](uint32_t key, int m, float2 a, float2 b) {
-                          const float t = __fdiv_rn(c.ys[m] - a.y, b.y - a.y);
-                          const uint32_t left = atomicSub(hist + key, 1u);
-                          xs[start[key] + left - 1] = order_of(fmaf(t, b.x - a.x, a.x));
-                      });
+                            uint32_t* __restrict__ xs, uint32_t* __restrict__ keys) {
+    const uint32_t lane = threadIdx.x & 31;
+    each_crossing(xy, loop_off, loop_of, layer_of, c,
+                  [&](uint32_t key, int m, float2 a, float2 b, uint32_t peers) {
+                      const float t = __fdiv_rn(c.ys[m] - a.y, b.y - a.y);
+                      const float x = fmaf(t, b.x - a.x, a.x);
+                      const int first = __ffs(peers) - 1;
+                      uint32_t left = 0;
+                      if (lane == (uint32_t)first)
+                          left = atomicSub(hist + key, (uint32_t)__popc(peers));
+                      left = __shfl_sync(peers, left, first);
+                      const int64_t at =
+                          start[key] + left - 1 - __popc(peers & ((1u << lane) - 1u));
+                      xs[at] = keys ? __float_as_uint(x) : order_of(x);
+                      if (keys) keys[at] = key;
+                  });
 }
 
 // A warp per line: its crossings sorted in shared memory (a bitonic network over
 // the next power of two, at most `room`) and its segments written in toolpath
 // order. 250 layers of 500 lines: 0.23 ms, bound by the latency of the loads and
 // stages (strides below 32 by shuffles instead: the same); the infill with the
-// counts (0.24 ms) and the buckets (0.36 ms) 0.84 ms, 1.39 ms with 7 passes of
-// radix sorts.
+// counts (0.22 ms) and the buckets (0.37 ms) 0.84 ms, 1.39 ms with 7 passes of
+// radix sorts. 1000 x 1000 squares x 3 layers (2,000 crossings per line): 0.90 ms, 1.68
+// with radix sorts alone; 3000 x 1000 (6,000 per line): buckets and radix sorts
+// 1.50 ms, 1.67 with radix sorts alone.
 constexpr int kLineMost = 2048, kLineWarps = 4;
+// Contours with as many vertices per line as this go straight to the radix sorts:
+// their lines are too long in all but odd cases, and so few counters are contended
+// (200,000 x 5 squares, 20 lines: 0.69 ms so, 4.4 ms with the lines counted first by an
+// atomic per crossing).
+constexpr uint64_t kLineVerts = 1 << 15;
 __global__ void __launch_bounds__(32 * kLineWarps)
 k_line_sort(const uint32_t* __restrict__ xs, const int64_t* __restrict__ start, int64_t n_keys,
             int64_t n_rec, int room, HatchConst c, float* __restrict__ out) {
@@ -384,7 +440,7 @@ csl_status csl_hatch_layers(const csl_contours* ct, double y0, double spacing, i
             CSL_LAUNCH_CHECK("hatch layer of loop");
             // the first loops may precede the first layer start only when layer 0
             // has loops; layer_loop_off[0] is 0, so the counts are the layers
-            if (n_keys <= (uint64_t)n_verts) {
+            if (n_keys <= (uint64_t)n_verts && (uint64_t)n_verts / n_keys < kLineVerts) {
                 DevBuf hist((size_t)n_keys * 4, s);
                 CSL_CUDA(cudaMemsetAsync(hist.get(), 0, (size_t)n_keys * 4, s));
                 k_line_count<<<grid_for(n_verts, 256), 256, 0, s>>>(
@@ -406,15 +462,16 @@ csl_status csl_hatch_layers(const csl_contours* ct, double y0, double spacing, i
                 if (h[2]) fail(CSL_ERR_CUDA, "hatching: a line with an odd number of crossings");
                 line_most = (int)std::min<uint32_t>(h[3], kLineMost + 1);
                 by_line = line_most <= kLineMost;
-                if (by_line && n_rec) {
+                if (n_rec) {
                     xs.alloc((size_t)n_rec * 4, s);
+                    if (!by_line) key.alloc((size_t)n_rec * 4, s);
                     k_line_emit<<<grid_for(n_verts, 256), 256, 0, s>>>(
                         xy, ct->loop_vert_off, loop_of.as<uint32_t>(), layer_of.as<uint32_t>(), c,
-                        line_start.as<int64_t>(), hist.as<uint32_t>(), xs.as<uint32_t>());
+                        line_start.as<int64_t>(), hist.as<uint32_t>(), xs.as<uint32_t>(),
+                        by_line ? nullptr : key.as<uint32_t>());
                     CSL_LAUNCH_CHECK("hatch line crossings");
                 }
-            }
-            if (!by_line) {
+            } else {
                 DevBuf cnt((size_t)n_verts * 4, s), pos((size_t)n_verts * 8, s);
                 k_count<<<grid_for(n_verts, 256), 256, 0, s>>>(xy, ct->loop_vert_off,
                                                                loop_of.as<uint32_t>(), c,
