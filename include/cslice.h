@@ -401,7 +401,8 @@ typedef struct csl_batch_opts {
     int32_t autotune;         /* nonzero: time the candidates (field kernel and tile, slab,
                                  CTAs per SM, staging chunk) and keep the fastest          */
     int32_t slab;             /* without autotune: 0 (8, or less for short jobs) or 2, 4, 8 */
-    int32_t ctas_per_sm;      /* without autotune: 0 (4) or 1 .. 6                     */
+    int32_t ctas_per_sm;      /* without autotune: 0 (4) or 1 .. 6; 4 at most where every
+                                 job's R is 10 pixels or more (more do not fit an SM)      */
     int32_t branches;         /* parallel graph branches for binner and contours: 0 (8) or 1 .. 32 */
     int32_t field_kernel;     /* without autotune: CSL_FIELD_AUTO (the block kernel),
                                  CSL_FIELD_BLOCK or CSL_FIELD_FOOTPRINT                 */
@@ -415,7 +416,7 @@ typedef struct csl_batch_opts {
 typedef struct csl_batch_info {
     int32_t n_jobs;
     int32_t slab;             /* chosen slab depth                                       */
-    int32_t ctas_per_sm;      /* chosen persistent CTAs per SM                           */
+    int32_t ctas_per_sm;      /* persistent CTAs per SM, in units of 256 threads         */
     int32_t from_cache;       /* 1: the choice came from the per-process cache           */
     int64_t n_items;          /* (job, slab, tile) items of the field queue              */
     int64_t n_pairs;          /* binner entries over all jobs                            */

@@ -164,7 +164,7 @@ void plan_jobs(csl_batch* b, int S, int kernel, int T, int K) {
     for (auto& J : b->jobs)
         fj.push_back(FieldBatchJob{J.L, J.g, &J.bins, J.sigma, J.mask, b->flag_d.as<uint32_t>()});
     field_batch_prepare(fj, b->fb, b->st);
-    field_batch_run(b->fb, b->n_sm * b->ctas, b->st);
+    field_batch_run(b->fb, b->n_sm, b->ctas, b->st);
     for (auto& J : b->jobs) {
         Replay rp{false, &J.plan, flag};
         contours_chunk(J.g, J.L->C, J.sigma, J.mask, J.want_eid, J.cont, b->st, &rp);
@@ -216,7 +216,7 @@ void capture(csl_batch* b, int ctas) {
         }
         join(b, 0);
         CSL_CUDA(cudaMemsetAsync(b->mask_arena.get(), 0, (size_t)b->mask_arena_words * 4, b->st));
-        field_batch_run(b->fb, b->n_sm * ctas, b->st);
+        field_batch_run(b->fb, b->n_sm, ctas, b->st);
         fork(b, K + 1);
         for (size_t j = 0; j < b->jobs.size(); ++j) {
             auto& J = b->jobs[j];
@@ -238,7 +238,7 @@ void capture(csl_batch* b, int ctas) {
     size_t n = 0;
     CSL_CUDA(cudaGraphGetNodes(b->graph, nullptr, &n));
     b->info.graph_nodes = (int64_t)n;
-    b->ctas = ctas;
+    b->ctas = std::min(ctas, field_batch_most_ctas(b->fb));
 }
 
 void launch_and_check(csl_batch* b, cudaStream_t s) {
@@ -396,6 +396,7 @@ csl_status csl_batch_create(csl_lattice* const* lats, const csl_slice_desc* desc
                 auto try_one = [&](int s_, int c_, int k_, int t_, int K_) {
                     plan(s_, k_, t_, K_);
                     capture(b, c_);
+                    c_ = b->ctas;
                     const float ms = time_graph(b);
                     if (nc < CSL_BATCH_MAX_CANDIDATES) {
                         b->info.cand_slab[nc] = s_;
@@ -420,9 +421,11 @@ csl_status csl_batch_create(csl_lattice* const* lats, const csl_slice_desc* desc
                 const int slabs[3] = {2, 4, 8};
                 for (int si = 0; si < 3; ++si) {
                     if (slabs[si] > min_layers && slabs[si] != 2) continue;
-                    const int cand_c[3] = {2, 4, 6};
+                    // (two pixel rows per thread: no more than 4 fit)
+                    const int cand_c[3] = {2, 4, b->fb.rows == 2 ? 3 : 6};
                     for (int ci = 0; ci < 3; ++ci) {
-                        if (k1.kernel == CSL_FIELD_FOOTPRINT && cand_c[ci] > 4) continue;
+                        if (k1.kernel == CSL_FIELD_FOOTPRINT && (cand_c[ci] & 1 || cand_c[ci] > 4))
+                            continue;
                         if (slabs[si] == S0 && cand_c[ci] == 4) continue;   // timed in step 1
                         try_one(slabs[si], cand_c[ci], k1.kernel, k1.T, 256);
                     }

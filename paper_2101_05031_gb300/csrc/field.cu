@@ -270,9 +270,10 @@ static_assert(sizeof(FieldJob) % 4 == 0, "FieldJob is copied as 32-bit words");
 
 // Persistent field kernel over the (job, slab, tile) items of a batch: each
 // CTA takes the next item from a shared counter, in the order `order` gives
-// (longest tile lists first, so the short ones fill the tail).
-template <int S, int PX>
-__global__ void __launch_bounds__(kFieldThreads / PX, 6)
+// (longest tile lists first, so the short ones fill the tail). CTAS: how many of
+// them an SM must hold (field_batch_run).
+template <int S, int PX, int CTAS>
+__global__ void __launch_bounds__(kFieldThreads / PX, CTAS)
 k_field_batch(const FieldJob* __restrict__ jobs, const uint2* __restrict__ items,
               const uint32_t* __restrict__ order, uint32_t n_items, uint32_t* counter) {
     __shared__ uint32_t s_item;
@@ -537,7 +538,13 @@ void field_batch_prepare(const std::vector<FieldBatchJob>& jobs, FieldBatch& fb,
     CSL_CUDA(cudaStreamSynchronize(s));   // the host tables above go out of scope
 }
 
-void field_batch_run(FieldBatch& fb, int n_ctas, cudaStream_t s) {
+int field_batch_most_ctas(const FieldBatch& fb) {
+    return fb.kernel == kFieldBlock && fb.rows == 2 ? 4 : 6;
+}
+
+void field_batch_run(FieldBatch& fb, int n_sm, int ctas, cudaStream_t s) {
+    ctas = std::min(ctas, field_batch_most_ctas(fb));
+    const int n_ctas = n_sm * ctas;
     if (fb.n_items == 0) return;
     const uint32_t n = (uint32_t)fb.n_items;
     k_item_keys<<<grid_for(fb.n_items, 256), 256, 0, s>>>(
@@ -555,15 +562,20 @@ void field_batch_run(FieldBatch& fb, int n_ctas, cudaStream_t s) {
         fp_batch_launch(fb.fp_jobs.get(), items, order, n, counter, fb.T, fb.S, fb.K, n_ctas, s);
         return;
     }
-    // with two pixel rows per thread a CTA has half the threads: twice as many CTAs
+    // With two pixel rows per thread a CTA has half the threads: twice as many CTAs, 8
+    // per SM at most, so 4 in the units of `ctas`. Registers for 8 of them (64 each)
+    // where they are wanted, else for 6 (79), which are a little faster while they are
+    // all there are: 12 batched lattices, S = 8, with 2, 3 and 4 per SM: 9.72, 8.45
+    // and 8.45 ms for 6 (the fourth did not fit), 9.86, 8.60 and 8.23 for 8. Room for 10
+    // or 12 costs spills: 8.46 and 8.61 ms at 6 per SM.
+#define CSL_FIELD_LAUNCH(SV, PXV, CT)                                                          \
+    k_field_batch<SV, PXV, CT><<<PXV * n_ctas, kFieldThreads / PXV, 0, s>>>(jobs, items, order, \
+                                                                            n, counter)
 #define CSL_FIELD_CASE(SV)                                                                     \
     case SV:                                                                                   \
-        if (fb.rows == 2)                                                                      \
-            k_field_batch<SV, 2><<<2 * n_ctas, kFieldThreads / 2, 0, s>>>(jobs, items, order,  \
-                                                                          n, counter);         \
-        else                                                                                   \
-            k_field_batch<SV, 1><<<n_ctas, kFieldThreads, 0, s>>>(jobs, items, order, n,       \
-                                                                  counter);                    \
+        if (fb.rows == 2 && ctas > 3) CSL_FIELD_LAUNCH(SV, 2, 8);                              \
+        else if (fb.rows == 2) CSL_FIELD_LAUNCH(SV, 2, 6);                                     \
+        else CSL_FIELD_LAUNCH(SV, 1, 6);                                                       \
         break;
     switch (fb.S) {
         CSL_FIELD_CASE(1)
@@ -573,6 +585,7 @@ void field_batch_run(FieldBatch& fb, int n_ctas, cudaStream_t s) {
         default: fail(CSL_ERR_INVALID_ARG, "slab depth must be 1, 2, 4 or 8");
     }
 #undef CSL_FIELD_CASE
+#undef CSL_FIELD_LAUNCH
     CSL_LAUNCH_CHECK("batch field");
 }
 

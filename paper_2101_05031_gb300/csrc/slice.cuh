@@ -131,9 +131,11 @@ void fp_batch_jobs(const std::vector<FieldBatchJob>& jobs, const float2* const* 
                    std::vector<unsigned char>& host);
 void fp_batch_launch(const void* jobs, const uint2* items, const uint32_t* order, uint32_t n,
                      uint32_t* counter, int T, int S, int K, int n_ctas, cudaStream_t s);
-// The run itself: queue order, counter reset, persistent launch of n_ctas
-// CTAs; reads nothing back (capturable in a CUDA graph).
-void field_batch_run(FieldBatch& fb, int n_ctas, cudaStream_t s);
+// The most CTAs of kFieldThreads threads per SM that the jobs' kernel is built for.
+int field_batch_most_ctas(const FieldBatch& fb);
+// The run itself: queue order, counter reset, persistent launch of `ctas` CTAs (that
+// many at most) on each of n_sm SMs; reads nothing back (capturable in a CUDA graph).
+void field_batch_run(FieldBatch& fb, int n_sm, int ctas, cudaStream_t s);
 
 // Contours of the chunk's layers (device arrays, layer-local edge ids).
 struct ChunkContours {
