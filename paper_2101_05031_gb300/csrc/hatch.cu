@@ -138,14 +138,15 @@ __device__ __forceinline__ float float_of(uint32_t k) {
 // of them instead of one per crossing takes 0.10 ms instead of 1.25 for the counts
 // of 3000 x 1000 squares (12 million crossings on 2,000 lines), which one address
 // after another had held up. Edges of more than kWideEdge lines are taken by all
-// lanes together.
-constexpr int kWideEdge = 32;
-template <class F>
+// lanes together, those of more than kLongEdge are only handed to long_edge(v, lines):
+// for the whole grid (each_long_crossing).
+constexpr int kWideEdge = 32, kLongEdge = 1024;
+template <class F, class G>
 __device__ __forceinline__ void each_crossing(const float2* __restrict__ xy,
                                               const int64_t* __restrict__ loop_off,
                                               const uint32_t* __restrict__ loop_of,
                                               const uint32_t* __restrict__ layer_of,
-                                              const HatchConst& c, F f) {
+                                              const HatchConst& c, F f, G long_edge) {
     const int lane = threadIdx.x & 31;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t v0 = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31u); v0 < c.n_verts;
@@ -164,6 +165,10 @@ __device__ __forceinline__ void each_crossing(const float2* __restrict__ xy,
                 m = first_line_at_or_above(c.ys, c.y0f, c.inv_sp, c.n_lines, lo);
                 m1 = first_line_at_or_above(c.ys, c.y0f, c.inv_sp, c.n_lines, hi);
                 base = layer_of[loop_of[v]] * (uint32_t)c.n_lines;
+                if (m1 - m > kLongEdge) {
+                    long_edge(v, m1 - m);
+                    m1 = m;
+                }
             }
         }
         uint32_t wide = __ballot_sync(0xffffffffu, m1 - m > kWideEdge);
@@ -175,8 +180,7 @@ __device__ __forceinline__ void each_crossing(const float2* __restrict__ xy,
                                          __shfl_sync(0xffffffffu, b.y, src));
             const uint32_t pb = __shfl_sync(0xffffffffu, base, src);
             const int from = __shfl_sync(0xffffffffu, m, src), to = __shfl_sync(0xffffffffu, m1, src);
-            for (int64_t k = from + lane; k < to; k += 32)
-                f(pb + (uint32_t)k, (int)k, p, q, 1u << lane);
+            for (int k = from + lane; k < to; k += 32) f(pb + (uint32_t)k, k, p, q, 1u << lane);
             if (lane == src) m = m1;
             __syncwarp();
         }
@@ -191,16 +195,65 @@ __device__ __forceinline__ void each_crossing(const float2* __restrict__ xy,
     }
 }
 
-// Crossings per line.
+// The crossings of the n listed pieces {vertex, piece of kLongEdge lines}, a block
+// each: one side of 100,000 lines in a lane (or a warp) is a chain of as many steps
+// (or a 32nd); 200 sides of 40,000 lines beside 30,000 squares: 1.04 ms, 17.4 with a warp
+// per side, 10.3 with radix sorts alone and a lane per side. f as above, each lane at a
+// line of its own.
+constexpr int kLongBlocks = 152 * 8;
+template <class F>
+__device__ __forceinline__ void each_long_crossing(const float2* __restrict__ xy,
+                                                   const int64_t* __restrict__ loop_off,
+                                                   const uint32_t* __restrict__ loop_of,
+                                                   const uint32_t* __restrict__ layer_of,
+                                                   const HatchConst& c,
+                                                   const uint2* __restrict__ list, uint32_t n,
+                                                   F f) {
+    for (uint32_t i = blockIdx.x; i < n; i += gridDim.x) {
+        const uint2 e = list[i];
+        const int64_t v = e.x;
+        int64_t w;
+        edge_of(loop_off, loop_of, v, w);
+        const float2 a = xy[v], b = xy[w];
+        const int m0 = first_line_at_or_above(c.ys, c.y0f, c.inv_sp, c.n_lines, fminf(a.y, b.y));
+        const int m1 = first_line_at_or_above(c.ys, c.y0f, c.inv_sp, c.n_lines, fmaxf(a.y, b.y));
+        const uint32_t base = layer_of[loop_of[v]] * (uint32_t)c.n_lines;
+        const int64_t from = m0 + (int64_t)e.y * kLongEdge;
+        const int64_t to = min((int64_t)m1, from + kLongEdge);
+        for (int64_t m = from + threadIdx.x; m < to; m += blockDim.x)
+            f(base + (uint32_t)m, (int)m, a, b, 1u << (threadIdx.x & 31));
+    }
+}
+
+// Crossings per line; the pieces of long edges are listed (n_list[0], room for `cap` of
+// them: more have more crossings together than the call takes, n_list[1]).
 __global__ void k_line_count(const float2* __restrict__ xy, const int64_t* __restrict__ loop_off,
                              const uint32_t* __restrict__ loop_of,
                              const uint32_t* __restrict__ layer_of, HatchConst c,
-                             uint32_t* __restrict__ hist) {
+                             uint32_t* __restrict__ hist, uint2* __restrict__ list,
+                             uint32_t cap, uint32_t* __restrict__ n_list) {
     const uint32_t lane = threadIdx.x & 31;
-    each_crossing(xy, loop_off, loop_of, layer_of, c,
-                  [&](uint32_t key, int, float2, float2, uint32_t peers) {
-                      if (lane == __ffs(peers) - 1u) atomicAdd(hist + key, (uint32_t)__popc(peers));
-                  });
+    each_crossing(
+        xy, loop_off, loop_of, layer_of, c,
+        [&](uint32_t key, int, float2, float2, uint32_t peers) {
+            if (lane == __ffs(peers) - 1u) atomicAdd(hist + key, (uint32_t)__popc(peers));
+        },
+        [&](int64_t v, int lines) {
+            const uint32_t n = ((uint32_t)lines + kLongEdge - 1u) / kLongEdge;
+            const uint32_t at = atomicAdd(n_list, n);
+            if (at >= cap || n > cap - at) atomicOr(n_list + 1, 1u);
+            for (uint32_t k = 0; k < n && at + k < cap; ++k) list[at + k] = make_uint2((uint32_t)v, k);
+        });
+}
+
+__global__ void k_line_count_long(const float2* __restrict__ xy,
+                                  const int64_t* __restrict__ loop_off,
+                                  const uint32_t* __restrict__ loop_of,
+                                  const uint32_t* __restrict__ layer_of, HatchConst c,
+                                  uint32_t* __restrict__ hist, const uint2* __restrict__ list,
+                                  uint32_t cap, const uint32_t* __restrict__ n_list) {
+    each_long_crossing(xy, loop_off, loop_of, layer_of, c, list, min(*n_list, cap),
+                       [&](uint32_t key, int, float2, float2, uint32_t) { atomicAdd(hist + key, 1u); });
 }
 
 // most[0] = the longest line's crossings; a line with an odd count is reported.
@@ -223,26 +276,47 @@ __global__ void k_line_most(const uint32_t* __restrict__ hist, int64_t n_keys,
 // Each crossing's x into its line's bucket: the slots left are counted down in
 // hist, which ends at 0. With keys (lines too long for a warp) the crossings' lines
 // beside them, and x as it is.
+struct LineBuckets {
+    const int64_t* __restrict__ start;
+    uint32_t* __restrict__ hist;
+    uint32_t* __restrict__ xs;
+    uint32_t* __restrict__ keys;
+
+    __device__ __forceinline__ void put(const HatchConst& c, uint32_t key, int m, float2 a,
+                                        float2 b, uint32_t peers) const {
+        const uint32_t lane = threadIdx.x & 31;
+        const float t = __fdiv_rn(c.ys[m] - a.y, b.y - a.y);
+        const float x = fmaf(t, b.x - a.x, a.x);
+        const int first = __ffs(peers) - 1;
+        uint32_t left = 0;
+        if (lane == (uint32_t)first) left = atomicSub(hist + key, (uint32_t)__popc(peers));
+        left = __shfl_sync(peers, left, first);
+        const int64_t at = start[key] + left - 1 - __popc(peers & ((1u << lane) - 1u));
+        xs[at] = keys ? __float_as_uint(x) : order_of(x);
+        if (keys) keys[at] = key;
+    }
+};
+
 __global__ void k_line_emit(const float2* __restrict__ xy, const int64_t* __restrict__ loop_off,
                             const uint32_t* __restrict__ loop_of,
-                            const uint32_t* __restrict__ layer_of, HatchConst c,
-                            const int64_t* __restrict__ start, uint32_t* __restrict__ hist,
-                            uint32_t* __restrict__ xs, uint32_t* __restrict__ keys) {
-    const uint32_t lane = threadIdx.x & 31;
-    each_crossing(xy, loop_off, loop_of, layer_of, c,
-                  [&](uint32_t key, int m, float2 a, float2 b, uint32_t peers) {
-                      const float t = __fdiv_rn(c.ys[m] - a.y, b.y - a.y);
-                      const float x = fmaf(t, b.x - a.x, a.x);
-                      const int first = __ffs(peers) - 1;
-                      uint32_t left = 0;
-                      if (lane == (uint32_t)first)
-                          left = atomicSub(hist + key, (uint32_t)__popc(peers));
-                      left = __shfl_sync(peers, left, first);
-                      const int64_t at =
-                          start[key] + left - 1 - __popc(peers & ((1u << lane) - 1u));
-                      xs[at] = keys ? __float_as_uint(x) : order_of(x);
-                      if (keys) keys[at] = key;
-                  });
+                            const uint32_t* __restrict__ layer_of, HatchConst c, LineBuckets to) {
+    each_crossing(
+        xy, loop_off, loop_of, layer_of, c,
+        [&](uint32_t key, int m, float2 a, float2 b, uint32_t peers) {
+            to.put(c, key, m, a, b, peers);
+        },
+        [](int64_t, int) {});
+}
+
+__global__ void k_line_emit_long(const float2* __restrict__ xy,
+                                 const int64_t* __restrict__ loop_off,
+                                 const uint32_t* __restrict__ loop_of,
+                                 const uint32_t* __restrict__ layer_of, HatchConst c,
+                                 LineBuckets to, const uint2* __restrict__ list, uint32_t n) {
+    each_long_crossing(xy, loop_off, loop_of, layer_of, c, list, n,
+                       [&](uint32_t key, int m, float2 a, float2 b, uint32_t peers) {
+                           to.put(c, key, m, a, b, peers);
+                       });
 }
 
 // A warp per line: its crossings sorted in shared memory (a bitonic network over
@@ -420,11 +494,12 @@ csl_status csl_hatch_layers(const csl_contours* ct, double y0, double spacing, i
 
         int64_t n_rec = 0;
         const uint64_t n_keys = (uint64_t)n_layers * (uint64_t)(n_lines > 0 ? n_lines : 1);
-        // small: [0, 1] crossings, [2] status, [3] the longest line's crossings
-        DevBuf key, xs, line_start, small(16, s);
+        // small: [0, 1] crossings, [2] status, [3] the longest line's crossings, [4] pieces of
+        // long edges, [5] more than their list holds
+        DevBuf key, xs, line_start, small(32, s);
         bool by_line = false;
         int line_most = 0;
-        CSL_CUDA(cudaMemsetAsync(small.get(), 0, 16, s));
+        CSL_CUDA(cudaMemsetAsync(small.get(), 0, 32, s));
         if (n_verts > 0 && n_lines > 0) {
             // loop of every vertex, layer of every loop
             DevBuf loop_of((size_t)n_verts * 4, s);
@@ -443,10 +518,24 @@ csl_status csl_hatch_layers(const csl_contours* ct, double y0, double spacing, i
             if (n_keys <= (uint64_t)n_verts && (uint64_t)n_verts / n_keys < kLineVerts) {
                 DevBuf hist((size_t)n_keys * 4, s);
                 CSL_CUDA(cudaMemsetAsync(hist.get(), 0, (size_t)n_keys * 4, s));
+                // pieces of long edges: at least half of each is lines that it crosses, so
+                // this many hold all the crossings that a call may have
+                const int64_t pieces = ceil_div(n_lines, kLongEdge);
+                const uint32_t long_cap = n_lines <= kLongEdge ? 0u
+                    : (uint32_t)std::min<int64_t>(n_verts * pieces, (2ll << 32) / kLongEdge);
+                DevBuf long_edges((size_t)std::max(long_cap, 1u) * 8, s);
                 k_line_count<<<grid_for(n_verts, 256), 256, 0, s>>>(
                     xy, ct->loop_vert_off, loop_of.as<uint32_t>(), layer_of.as<uint32_t>(), c,
-                    hist.as<uint32_t>());
+                    hist.as<uint32_t>(), long_edges.as<uint2>(), long_cap,
+                    small.as<uint32_t>() + 4);
                 CSL_LAUNCH_CHECK("hatch line counts");
+                if (long_cap) {
+                    k_line_count_long<<<kLongBlocks, 256, 0, s>>>(
+                        xy, ct->loop_vert_off, loop_of.as<uint32_t>(), layer_of.as<uint32_t>(), c,
+                        hist.as<uint32_t>(), long_edges.as<uint2>(), long_cap,
+                        small.as<uint32_t>() + 4);
+                    CSL_LAUNCH_CHECK("hatch line counts of long edges");
+                }
                 k_line_most<<<grid_for((int64_t)n_keys, 256), 256, 0, s>>>(
                     hist.as<uint32_t>(), (int64_t)n_keys, small.as<uint32_t>() + 2,
                     small.as<uint32_t>() + 3);
@@ -454,10 +543,10 @@ csl_status csl_hatch_layers(const csl_contours* ct, double y0, double spacing, i
                 line_start.alloc((size_t)n_keys * 8, s);
                 exclusive_scan_u32_to_i64(hist.as<uint32_t>(), line_start.as<int64_t>(),
                                           (int64_t)n_keys, small.as<int64_t>(), s);
-                uint32_t h[4];
-                read_to_host(h, small.get(), 16, s);
+                uint32_t h[6];
+                read_to_host(h, small.get(), sizeof h, s);
                 n_rec = (int64_t)(((uint64_t)h[1] << 32) | h[0]);
-                if (n_rec >= 0xffffffffLL) fail(CSL_ERR_CAPACITY, "too many crossings");
+                if (n_rec >= 0xffffffffLL || h[5]) fail(CSL_ERR_CAPACITY, "too many crossings");
                 if (n_rec % 2) fail(CSL_ERR_CUDA, "hatching: odd number of crossings");
                 if (h[2]) fail(CSL_ERR_CUDA, "hatching: a line with an odd number of crossings");
                 line_most = (int)std::min<uint32_t>(h[3], kLineMost + 1);
@@ -465,11 +554,18 @@ csl_status csl_hatch_layers(const csl_contours* ct, double y0, double spacing, i
                 if (n_rec) {
                     xs.alloc((size_t)n_rec * 4, s);
                     if (!by_line) key.alloc((size_t)n_rec * 4, s);
+                    const LineBuckets to{line_start.as<int64_t>(), hist.as<uint32_t>(),
+                                         xs.as<uint32_t>(), by_line ? nullptr : key.as<uint32_t>()};
                     k_line_emit<<<grid_for(n_verts, 256), 256, 0, s>>>(
                         xy, ct->loop_vert_off, loop_of.as<uint32_t>(), layer_of.as<uint32_t>(), c,
-                        line_start.as<int64_t>(), hist.as<uint32_t>(), xs.as<uint32_t>(),
-                        by_line ? nullptr : key.as<uint32_t>());
+                        to);
                     CSL_LAUNCH_CHECK("hatch line crossings");
+                    if (h[4]) {
+                        k_line_emit_long<<<kLongBlocks, 256, 0, s>>>(
+                            xy, ct->loop_vert_off, loop_of.as<uint32_t>(), layer_of.as<uint32_t>(),
+                            c, to, long_edges.as<uint2>(), h[4]);
+                        CSL_LAUNCH_CHECK("hatch line crossings of long edges");
+                    }
                 }
             } else {
                 DevBuf cnt((size_t)n_verts * 4, s), pos((size_t)n_verts * 8, s);

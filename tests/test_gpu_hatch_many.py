@@ -20,6 +20,10 @@ def _rows(per_row, rows, height):
     ([np.concatenate([_rows(300, 20, 0.6), _rows(5, 1, 33.0) - [7.5, 0, 0, 0]])] * 2, 500, 0.07),
     ([_rows(1100, 1, 30.0)], 90, 0.31),               # long lines, sides of 97 lines
     ([_rows(9000, 1, 0.6)], 1, 0.3),                  # 36,000 vertices for one line
+    # sides of 1024, 1025, 2049 and 3,300 lines beside short ones; in lines too long for a warp
+    ([np.concatenate([_rows(40, 60, 0.6), [[-2, 0, 0.5, 30.705], [-4, 0, 0.5, 30.735],
+                                           [-6, 3, 0.5, 61.455], [-8, 0, 0.5, 99.0]]])] * 2, 3400, 0.03),
+    ([np.concatenate([_rows(1100, 1, 30.0), [[-2, 0.0, 0.5, 12.0]]])], 1300, 0.02),
     ([_rows(40, 30, 0.6), _rows(1, 1, 0.6)[:0], _rows(1, 1, 31.0)], 100, 0.3),   # an empty layer
 ])
 def test_rows(parts, n_lines, sp):
