@@ -179,8 +179,10 @@ __device__ __forceinline__ void each_crossing(const float2* __restrict__ xy,
             const float2 q = make_float2(__shfl_sync(0xffffffffu, b.x, src),
                                          __shfl_sync(0xffffffffu, b.y, src));
             const uint32_t pb = __shfl_sync(0xffffffffu, base, src);
-            const int from = __shfl_sync(0xffffffffu, m, src), to = __shfl_sync(0xffffffffu, m1, src);
-            for (int k = from + lane; k < to; k += 32) f(pb + (uint32_t)k, k, p, q, 1u << lane);
+            const int from = __shfl_sync(0xffffffffu, m, src);
+            const int n = __shfl_sync(0xffffffffu, m1, src) - from;
+            for (int k = lane; k < n; k += 32)
+                f(pb + (uint32_t)(from + k), from + k, p, q, 1u << lane);
             if (lane == src) m = m1;
             __syncwarp();
         }
