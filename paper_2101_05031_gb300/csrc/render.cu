@@ -378,9 +378,14 @@ extern "C" csl_status csl_render_depth(const csl_lattice* L, const csl_camera* c
         // shorten the lists that a sample sums and make more pairs to sort
         // (429,039 struts of about 1 mm, R = 0.525 mm, 1920 x 1080 rays: cells of
         // 0.75, 1, 1.3 and 1.6 R take 5.3, 4.5, 4.2 and 4.3 ms, of which the rays
-        // 2.7, 3.1, 3.3 and 3.7 ms). Where that makes more than 2^27 strut-cell
-        // pairs (2 GB of lists) the edge is doubled, and again while there are
-        // 2^31 pairs.
+        // 2.7, 3.1, 3.3 and 3.7 ms). Where that makes many pairs for the pixels the
+        // sort costs more than the rays, and the cells are of 2 R: above 2^23 pairs and 64
+        // for each pixel, where no lattice timed lost by it (3.5 million struts, 64 x 48
+        // rays: 3.6 ms, 5.9 with cells of 1.3 R, 5.0 with cells of 2 R by bounding
+        // boxes; 1280 x 720: 5.6, 7.4 and 10.0; 1 million short struts, 320 x 240: 2.0, 2.2
+        // and 2.9, but 640 x 480: 3.3 and 3.1 ms). Where that makes
+        // more than 2^27 strut-cell pairs (2 GB of lists) the edge is doubled, and
+        // again while there are 2^31 pairs.
         RvGrid g;
         double scale = 1.0;
         for (int k = 0; k < 3; ++k)
@@ -390,8 +395,10 @@ extern "C" csl_status csl_render_depth(const csl_lattice* L, const csl_camera* c
         const csl_rec* rec = L->rec.as<csl_rec>();
         DevBuf d_cnt((size_t)ne * 4, s), d_off((size_t)ne * 8, s), d_tot(8, s);
         int64_t n_cells = 0, n_pairs = 0;
+        double base = 1.3 * R;
         for (int grow = 0;; ++grow) {
-            double h = std::max(ldexp(1.3 * R, grow), 1e-6);
+            double h = std::max(ldexp(base, grow), 1e-6);
+            const double want = h;
             int dims[3];
             auto dims_of = [&](double hh) {
                 double tot = 1;
@@ -418,6 +425,12 @@ extern "C" csl_status csl_render_depth(const csl_lattice* L, const csl_camera* c
             exclusive_scan_u32_to_i64(d_cnt.as<uint32_t>(), d_off.as<int64_t>(), ne,
                                       d_tot.as<int64_t>(), s);
             n_pairs = read_i64(d_tot.as<int64_t>(), s);
+            if (grow == 0 && n_pairs <= (1ll << 27) && h == want && base < 2.0 * R &&
+                n_pairs > (1ll << 23) + 64 * n_px) {
+                base = 2.0 * R;
+                grow = -1;
+                continue;
+            }
             if (n_pairs <= (1ll << 27) || (grow > 0 && n_pairs < (1ll << 31))) break;
             if (n_cells == 8) fail(CSL_ERR_CAPACITY, "more than 2^31 strut-cell pairs");
         }
