@@ -564,6 +564,15 @@ csl_status csl_debug_wait_timeout(uint32_t polls, void* stream);
 csl_status csl_debug_lattice_timeout(csl_lattice* lat, uint32_t polls, void* stream);
 
 /*
+ * csl_debug_sort_pairs -- the stable radix sort that orders struts, bins and
+ * lists, by itself: sorts n device pairs in place by the low key_bits bits
+ * (1 .. 32) of the keys, whose other bits are 0, equal keys in input order. For
+ * tests. The paper has no counterpart. Synchronises the stream.
+ */
+csl_status csl_debug_sort_pairs(uint32_t* keys, uint32_t* vals, int64_t n, int32_t key_bits,
+                                void* stream);
+
+/*
  * csl_measure_fp32_peak -- FP32 throughput of the device, measured with a
  * kernel of independent FFMA chains at full occupancy (best of 5 timed
  * launches after one warm-up). A measurement helper for the roofline of the

@@ -173,6 +173,7 @@ SIGNATURES = [
                                     ctypes.POINTER(c_f64), ctypes.POINTER(c_f64), c_vp]),
     ("csl_debug_wait_timeout", c_i32, [ctypes.c_uint32, c_vp]),
     ("csl_debug_lattice_timeout", c_i32, [c_vp, ctypes.c_uint32, c_vp]),
+    ("csl_debug_sort_pairs", c_i32, [c_vp, c_vp, c_i64, c_i32, c_vp]),
     ("csl_density_match", c_i32, [c_vp, c_i64, c_vp, c_i64, ctypes.POINTER(Voxels),
                                   ctypes.POINTER(DmParams), c_vp,
                                   ctypes.POINTER(ctypes.POINTER(DmResult))]),

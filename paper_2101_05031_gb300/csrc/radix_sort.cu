@@ -196,3 +196,23 @@ void radix_sort_pairs(uint32_t* keys, uint32_t* vals, uint32_t* tmp_keys, uint32
 }
 
 }  // namespace csl
+
+extern "C" csl_status csl_debug_sort_pairs(uint32_t* keys, uint32_t* vals, int64_t n,
+                                           int32_t key_bits, void* stream) {
+    try {
+        if (!keys || !vals || n < 0 || key_bits < 1 || key_bits > 32)
+            csl::fail(CSL_ERR_INVALID_ARG, "device arrays, n >= 0 and key_bits in [1, 32]");
+        cudaStream_t s = (cudaStream_t)stream;
+        const size_t bytes = (size_t)(n > 0 ? n : 1) * 4;
+        csl::DevBuf tk(bytes, s), tv(bytes, s);
+        csl::radix_sort_pairs(keys, vals, tk.as<uint32_t>(), tv.as<uint32_t>(), n, key_bits, s);
+        CSL_CUDA(cudaStreamSynchronize(s));
+        return CSL_OK;
+    } catch (const csl::Error& e) {
+        csl::set_last_error(e.what());
+        return e.code;
+    } catch (const std::exception& e) {
+        csl::set_last_error(e.what());
+        return CSL_ERR_CUDA;
+    }
+}
