@@ -121,7 +121,9 @@ __device__ float warp_bisect_ratio(const float* F, const float* J, int n, float 
     const float r_hi = warp_mean<false>(F, J, n, ends.hi, c);
     *rho_hi = r_hi;
     if (r_hi <= target) return 2.0f;
-    if (!warp_mean_below(F, J, n, ends.lo, target, c) && target == target) return 0.5f;
+    // (a mean or target that is no number is neither below nor at the other: halved)
+    if (r_hi == r_hi && target == target && !warp_mean_below(F, J, n, ends.lo, target, c))
+        return 0.5f;
     float lo = 0.5f, hi = 2.0f;
     for (int it = 0; it < c.iters; it += 5) {
         float a = lo, b = hi;
