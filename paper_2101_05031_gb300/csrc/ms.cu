@@ -307,78 +307,36 @@ __global__ void __launch_bounds__(32 * kEmitWarps, 12) k_emit(
 }
 
 // Each splitter walks its segment up to the next splitter (nxt: successor |
-// splitter bit, one 4-byte load per step). A walk is a chain of dependent
-// loads, so every thread advances kWalks walks of different segments in
-// lockstep: their loads are independent and in flight together.
-constexpr int kWalks = 1;
-
+// splitter bit, one 4-byte load per step), a thread per splitter: several walks in
+// lockstep per thread were no faster, the walks of the other warps hide the loads.
 __global__ void k_segments(const uint32_t* __restrict__ nxt,
                            const uint32_t* __restrict__ spos, const uint32_t* __restrict__ split_id,
                            int64_t ns, int64_t n, uint32_t* __restrict__ seg_next,
                            uint32_t* __restrict__ seg_len, uint32_t* status) {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t0 < ns;
-         t0 += stride * kWalks) {
-        uint32_t j[kWalks];
-        int64_t len[kWalks];
-        bool live[kWalks], bad[kWalks];
-#pragma unroll
-        for (int g = 0; g < kWalks; ++g) {
-            const int64_t t = t0 + g * stride;
-            live[g] = bad[g] = false;
-            len[g] = 1;
-            j[g] = 0;
-            if (t >= ns) continue;
-            const uint32_t s0 = split_id[t];
-            if ((int64_t)s0 >= n) {   // a replay whose sizes changed (flagged): no walk
-                bad[g] = true;
-                continue;
+    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < ns;
+         t += (int64_t)gridDim.x * blockDim.x) {
+        const uint32_t s0 = split_id[t];
+        // (beyond n: a replay whose sizes changed, flagged: no walk)
+        uint32_t j = (int64_t)s0 < n ? nxt[s0] & 0x7fffffffu : 0xffffffffu, sn = 0;
+        int64_t len = 1;
+        bool bad = true;
+        while ((int64_t)j < n && len <= n) {   // else corrupt links
+            const uint32_t v = nxt[j];
+            if (v >> 31) {   // the next splitter
+                sn = spos[j];
+                bad = (int64_t)sn >= ns;   // more splitters than planned (flagged)
+                break;
             }
-            j[g] = nxt[s0] & 0x7fffffffu;
-            live[g] = true;
+            j = v & 0x7fffffffu;
+            ++len;
         }
-        for (;;) {
-            bool any = false;
-            uint32_t v[kWalks];
-#pragma unroll
-            for (int g = 0; g < kWalks; ++g) {
-                if (live[g] && ((int64_t)j[g] >= n || len[g] > n)) {   // corrupt links
-                    live[g] = false;
-                    bad[g] = true;
-                }
-                v[g] = live[g] ? nxt[j[g]] : 0u;
-            }
-#pragma unroll
-            for (int g = 0; g < kWalks; ++g) {
-                if (!live[g]) continue;
-                if (v[g] >> 31) {   // the next splitter
-                    live[g] = false;
-                } else {
-                    j[g] = v[g] & 0x7fffffffu;
-                    ++len[g];
-                    any = true;
-                }
-            }
-            if (!any) break;
+        if (bad) {   // report, never loop forever
+            atomicOr(status, ST_CAPACITY);
+            sn = (uint32_t)t;
+            len = 1;
         }
-#pragma unroll
-        for (int g = 0; g < kWalks; ++g) {
-            const int64_t t = t0 + g * stride;
-            if (t >= ns) continue;
-            uint32_t sn = 0;
-            if (!bad[g]) {
-                sn = spos[j[g]];
-                if ((int64_t)sn >= ns) bad[g] = true;   // more splitters than planned (flagged)
-            }
-            if (bad[g]) {   // report, never loop forever
-                atomicOr(status, ST_CAPACITY);
-                seg_next[t] = (uint32_t)t;
-                seg_len[t] = 1;
-            } else {
-                seg_next[t] = sn;
-                seg_len[t] = (uint32_t)len[g];
-            }
-        }
+        seg_next[t] = sn;
+        seg_len[t] = (uint32_t)len;
     }
 }
 
