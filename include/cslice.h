@@ -341,7 +341,8 @@ csl_status csl_volume_fraction(csl_lattice* lat, const csl_cells* cells, float* 
 /*
  * csl_volume_fraction_backward -- gradient of a scalar loss L with respect to
  * every radius and node position, given grad_vf = dL/dvf (device, the layout
- * of vf_out). Sigma is recomputed (nothing is kept from the forward call).
+ * of vf_out). Sigma is recomputed (nothing is kept from the forward call), in the
+ * same device memory: 1 GiB, or one layer of cells' samples where that is more.
  *   dL/drho_j = sum_c grad_vf_c (1/m^3) sum_p s(1-s)/T * I_j(p) * dw_j/drho_j
  *   dL/dv_i   = sum over the edges at node i of the same factor times
  *               w_j dI_j/d(endpoint)

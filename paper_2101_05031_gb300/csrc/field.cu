@@ -22,8 +22,8 @@
 // records themselves, in list order), is staged into shared memory in chunks of
 // 256 records by one bulk copy (TMA, cp.async.bulk) completed on an mbarrier;
 // each thread converts its record to tile-local coordinates, then computes for
-// every (record, layer) item whether the edge's support can reach each warp's
-// 8x4-pixel block (xy box of the edge clipped to |z - z_layer| <= R, grown by
+// every (record, layer) item whether the edge's support can reach each warp's block
+// of 8x4 or 8x8 pixels (xy box of the edge clipped to |z - z_layer| <= R, grown by
 // R, and the block centre's distance to the line). Warps then walk only the
 // records whose bit is set (ballot + ffs); the per-pixel evaluation is
 // branch-free.
@@ -41,11 +41,8 @@ namespace {
 struct FieldConst {
     int32_t nx, ny, ntx, n_tiles;
     int32_t n_layers;      // layers in this chunk
-    int32_t first_layer;   // global index of the chunk's first layer
-    double x0, y0, px, z0, dz;
-    float R2, inv_R4, fpx, fdz, cull;
-    float cull_line2;   // (cull + half-diagonal of a warp's pixel block)^2
-    TileCull tc;        // the same values for stage_record
+    float R2, fpx, fdz;
+    TileCull tc;
     float C;            // iso-value (inside mask)
     const float2* org_x;   // per tile column: x of its first pixel edge, (hi, lo)
     const float2* org_y;   // per tile row
@@ -382,30 +379,21 @@ FieldConst make_field_const(const ChunkGeom& g, float C, const float2* org, int 
     c.ntx = g.ntx;
     c.n_tiles = g.ntx * g.nty;
     c.n_layers = g.n_layers;
-    c.first_layer = g.first_layer;
-    c.x0 = g.x0;
-    c.y0 = g.y0;
-    c.px = g.px;
-    c.z0 = g.z0;
-    c.dz = g.dz;
     c.R2 = (float)(g.R * g.R);
-    c.inv_R4 = (float)(1.0 / (g.R * g.R * g.R * g.R));
     c.fpx = (float)g.px;
     c.fdz = (float)g.dz;
-    c.cull = (float)(g.R * (1.0 + 1e-5) + 1e-6);
+    c.tc.cull = (float)(g.R * (1.0 + 1e-5) + 1e-6);
     {
         // pixel centres of a warp's block of 8 x 4 rows pixels lie within 3.5 x
         // (2 rows - 1/2) pixels of its centre
         const double hy = 2.0 * rows - 0.5;
         double hd = g.px * sqrt(3.5 * 3.5 + hy * hy) * (1.0 + 1e-5);
-        double r = (double)c.cull + hd;
-        c.cull_line2 = (float)(r * r);
+        double r = (double)c.tc.cull + hd;
+        c.tc.cull_line2 = (float)(r * r);
     }
     c.tc.fpx = c.fpx;
     c.tc.fdz = c.fdz;
-    c.tc.cull = c.cull;
-    c.tc.cull_line2 = c.cull_line2;
-    c.tc.inv_R4 = c.inv_R4;
+    c.tc.inv_R4 = (float)(1.0 / (g.R * g.R * g.R * g.R));
     return c;
 }
 

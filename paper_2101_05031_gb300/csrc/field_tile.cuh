@@ -8,7 +8,7 @@
 
 namespace csl {
 
-constexpr int kTileWarps = 8;   // a CTA = 8 warps, each an 8 x 4 pixel block
+constexpr int kTileWarps = 8;   // blocks of 8 x 4 pixels in a tile, a warp each (or for two)
 
 struct TileCull {
     float fpx, fdz;      // pixel size, layer spacing (float)
@@ -93,7 +93,6 @@ __device__ __forceinline__ uint32_t cull_layer(const float4 A, const float4 B, i
     const float zl = (float)l * c.fdz;
     float t_lo = 0.0f, t_hi = len;
     if (uz > 1e-12f) {
-        // approximate: these bounds move by far less than cull's slack
         const float inv_uz = 1.0f / uz;
         t_lo = fmaxf((zl - c.cull - az) * inv_uz, 0.0f);
         t_hi = fminf((zl + c.cull - az) * inv_uz, len);

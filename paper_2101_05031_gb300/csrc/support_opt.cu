@@ -6,16 +6,17 @@
 // inside the inscribed sphere of its star (Eq. 17). The paper visits the
 // vertices one by one; here a greedy colouring (vertex order, smallest colour
 // free among the neighbours) orders them colour by colour. Vertices of one
-// colour share no edge, so each colour is one kernel launch with a warp per
-// vertex, and the result equals the sequential sweep in that order.
+// colour share no edge, so each colour is one kernel launch with half a warp or a
+// warp per vertex, and the result equals the sequential sweep in that order.
 //
 // A move goes along -grad J by step * tau0 (tau0: the smallest distance from
 // the vertex's initial position o to the faces opposite it), halved up to
 // `backtracks` times until the position lies in the ball |p - o| <= ball *
 // tau0, every incident tetrahedron keeps its orientation and min_volume of its
-// initial volume, and J decreases. Rounds repeat until nothing moves. All
-// arithmetic is FP64 in one fixed order (the build compiles device code with
-// --fmad=false).
+// initial volume, and J decreases. Rounds repeat until nothing moves. Positions,
+// gradients and sums are FP64 in one fixed order (the build compiles device code
+// with --fmad=false); a trial's tests are screened in FP32 with error bounds and
+// decided in FP64 where those leave them open, so that the moves are those of FP64.
 #include <limits.h>
 #include <math.h>
 

@@ -479,6 +479,7 @@ void vf_backward(csl_lattice* L, const csl_cells& cells, const float* grad_vf, f
     const int cz = cells.dims[2];
     DevBuf acc((size_t)ne * 32, s);
     CSL_CUDA(cudaMemsetAsync(acc.get(), 0, (size_t)ne * 32, s));
+    // as much as the forward pass holds: 1 GiB, or one layer of cells where that is more
     DevBuf sigma((size_t)cells.dims[0] * cells.dims[1] * per * cells.m * cells.m * cells.m * 4, s);
     for (int first = 0; first < cz; first += per) {
         const int n = std::min(per, cz - first);
