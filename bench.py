@@ -33,33 +33,39 @@ METRIC = "pixel-evals/s and layers/s at 10M and 100M struts; backward/forward ti
 F_PAIR = 36            # FP32 flops of one (pixel, layer, edge) term in the field kernel
 # Per field kernel, from an ncu capture of one launch on a 1.6M-strut graded
 # lattice, 1000^2 px x 120 layers (profiles/): the FP32 instructions it executes
-# per cycle as a fraction of the FP32 peak (every evaluated lane), and its DRAM
-# bytes (read + write) per pixel-layer (scaled by pixel-layers to a launch of the
-# timed workload). None where no capture of the current kernel exists.
+# per cycle as a fraction of the FP32 peak (every evaluated lane). Its DRAM bytes
+# (read + write) per pixel-layer, scaled by pixel-layers to a launch of the timed
+# workload: the footprint kernel's from a launch of the 103M-strut lattice
+# itself, 4000^2 px x 64 layers (more than the smaller lattice's 4.31: records and
+# planes do not stay in L2), the block kernel's from the 1.6M-strut launch.
 NCU_FIELD = {
     "block": {"kernel": "k_field", "executed_frac": (2 * 2543.9 + 1367.4 + 2033.7) / (152 * 128 * 2),
               "dram_bytes_per_pixel_layer": (0.128309e9 + 0.435139e9) / (120 * 1000 * 1000),
               "profile": "profiles/field_kernels.txt"},
     "footprint": {"kernel": "k_field_fp",
                   "executed_frac": (2 * 2973.3 + 1293.7 + 1552.0) / (152 * 128 * 2),
-                  "dram_bytes_per_pixel_layer": (0.078409e9 + 0.438833e9) / (120 * 1000 * 1000),
+                  "dram_bytes_per_pixel_layer": (0.66177e9 + 4.15e9) / (64 * 4000 * 4000),
                   "profile": "profiles/field_kernels.txt"},
 }
 # The volume fraction's FP32 work beyond the field term: per sample, the
-# sigmoid and the mean (forward), the sigmoid and alpha (the adjoint's pass 1);
-# per term of the adjoint's pass 2 (coordinates, the clipped chord, the 3-point
-# moments M0..M2 and I, and the 7 partials), counting FMA as 2 and add, sub and
-# mul as 1, as written in its kernel.
+# sigmoid and the mean (forward), the sigmoid and alpha (the adjoint); per term
+# of the adjoint's gradients (coordinates, the clipped chord, the 3-point moments
+# M0..M2 and I, and the 7 partials), counting FMA as 2 and add, sub and mul as 1,
+# as written in its kernel.
 VF_FLOPS_PER_SAMPLE = 4
 VF_GRAD_FLOPS_PER_SAMPLE = 8
 VF_GRAD_FLOPS_PER_TERM = 124
 # Executed FP32 fractions of the volume-fraction kernels from one ncu capture
 # each on a Freudenthal lattice of 27^3 nodes, 32^3 cells x 8^3 samples: FFMA (2 flops), FADD and FMUL
-# thread instructions per cycle over the FP32 peak per cycle.
+# thread instructions per cycle over the FP32 peak per cycle. The backward pass
+# evaluates the field again (0.777 ms of that capture) before its own kernel
+# (0.40 ms): its fraction is theirs by time.
 NCU_VF = {"forward": {"kernel": "k_field",
                       "executed_frac": (2 * 4031.1 + 1949.8 + 3057.9) / (152 * 128 * 2)},
-          "backward": {"kernel": "k_vf_grad",
-                       "executed_frac": (2 * 341.7 + 620.1 + 314.7) / (152 * 128 * 2)},
+          "backward": {"kernel": "k_field, k_vf_grad",
+                       "executed_frac": (0.777 * (2 * 4031.1 + 1949.8 + 3057.9)
+                                         + 0.40 * (2 * 341.7 + 620.1 + 314.7))
+                       / (0.777 + 0.40) / (152 * 128 * 2)},
           "profile": "profiles/other_kernels.txt"}
 HBM_GBS = 6772.9       # measured copy bandwidth of the GPU
 # algorithmic bytes of the HBM-bound stages
@@ -308,11 +314,11 @@ def run_vf(steps, warmup):
     # pitch h/m whose layers lie every h/m from half a pitch above the origin,
     # so the slicing kernel's exact counting pass on that grid counts the
     # nonzero (sample, strut) terms the forward evaluates (36 flops each, plus
-    # the sigmoid and the mean per sample). The backward recomputes them (its
-    # pass 1) and then evaluates the moments and the 7 partials only where the
-    # sigmoid has not saturated, a thin shell around the iso-surface whose
-    # term count the library does not report: its algorithmic figure here is
-    # pass 1 alone (a lower bound), beside ncu's executed FP32 fraction.
+    # the sigmoid and the mean per sample). The backward evaluates the field again
+    # and then the moments and the 7 partials only where the sigmoid has not
+    # saturated, a thin shell around the iso-surface whose term count the library
+    # does not report: its algorithmic figure here is the field and alpha alone
+    # (a lower bound), beside ncu's executed FP32 fraction.
     m = cells["m"]
     pitch = cells["h"] / m
     lat.slice(z0=cells["origin"][2] + 0.5 * pitch, dz=pitch, n_layers=d[2] * m,
@@ -335,15 +341,15 @@ def run_vf(steps, warmup):
                      "peak": peak, "unit": "TFLOP/s",
                      "frac_lower_bound": f_bwd1 / (bwd / 1e3) / 1e12 / peak,
                      "flops_per_term_pass2": VF_GRAD_FLOPS_PER_TERM,
-                     "lower_bound_basis": "pass 1 only (Sigma recomputed: 36 flops per nonzero "
-                                          "term, sigmoid and alpha per sample); pass 2's "
+                     "lower_bound_basis": "the field evaluated again (36 flops per nonzero "
+                                          "term) and sigmoid and alpha per sample; the gradients' "
                                           f"{VF_GRAD_FLOPS_PER_TERM} flops per term where the "
                                           "sigmoid has not saturated are not counted",
                      "executed_frac_ncu": NCU_VF["backward"]["executed_frac"],
                      "executed_kernel": NCU_VF["backward"]["kernel"]},
         "peak_basis": "152 SMs x 128 FP32 lanes x 2 x 2070 MHz (max SM clock)",
-        "executed_basis": "ncu FFMA + FADD + FMUL thread instructions per cycle of one launch "
-                          f"({NCU_VF['profile']})"}
+        "executed_basis": "ncu FFMA + FADD + FMUL thread instructions per cycle of one launch of "
+                          f"each kernel, weighted by its time ({NCU_VF['profile']})"}
     # the FP64 oracle on a sample of 2 cells in the middle of the grid (one host core)
     import oracle
     n_cells = d[0] * d[1] * d[2]
@@ -801,8 +807,9 @@ def main():
             "frac": achieved / peak,
             "traffic": (ncu["dram_bytes_per_pixel_layer"] * px_layers_per_launch
                         if ncu["dram_bytes_per_pixel_layer"] else None),
-            "traffic_basis": "ncu dram bytes of one field launch on a 1.6M-strut graded "
-                             "lattice, scaled by pixel-layers per launch",
+            "traffic_basis": "ncu dram bytes of one field launch on a graded lattice (103M struts, "
+                             "4000^2 px x 64 layers; block kernel: 1.6M struts), scaled by "
+                             "pixel-layers per launch",
             "kernel": ncu["kernel"], "flops_per_term": F_PAIR,
             "nonzero_terms_per_step": pairs, "evaluated_terms_per_step": evaluated,
             "candidate_entries_per_step": cand,

@@ -402,7 +402,7 @@ FieldConst make_field_const(const ChunkGeom& g, float C, const float2* org, int 
 // against 1,151 million evaluated terms for 818 million nonzero ones at R = 26
 // px, with 17 % fewer instructions in all). Field of 2000^2 px x 200 layers at R
 // = 26 px: 20.4 ms with one row, 17.5 with two (90 % issue); at 15 px (12 batched
-// lattices) 8.0 and 6.8 ms, at 10.5 px (780^2 x 190) 4.11 and 3.91 ms. Below, one
+// lattices) 8.0 and 6.6 ms, at 10.5 px (780^2 x 190) 4.11 and 3.91 ms. Below, one
 // row: there the automatic choice takes the footprint kernel, and the volume
 // fraction's samples (R = 5 px) keep 8 x 4 blocks.
 int rows_per_thread(const ChunkGeom& g) { return g.R >= 10.0 * g.px ? 2 : 1; }

@@ -350,8 +350,9 @@ __global__ void k_line_emit_long(const float2* __restrict__ xy,
 // the next power of two, at most `room`) and its segments written in toolpath
 // order. 250 layers of 500 lines: 0.23 ms, bound by the latency of the loads and
 // stages (strides below 32 by shuffles instead: the same); the infill with the
-// counts (0.22 ms) and the buckets (0.37 ms) 0.84 ms, 1.39 ms with 7 passes of
-// radix sorts. 1000 x 1000 squares x 3 layers (2,000 crossings per line): 0.90 ms, 1.68
+// counts (0.19 ms) and the buckets (0.34 ms) 1.03 ms a call, 1.10 with an atomic per
+// crossing in both (0.23 and 0.35; 0.84 ms of kernels, where 7 passes of radix sorts
+// made 1.39). 1000 x 1000 squares x 3 layers (2,000 crossings per line): 0.90 ms, 1.68
 // with radix sorts alone; 3000 x 1000 (6,000 per line): buckets and radix sorts
 // 1.50 ms, 1.67 with radix sorts alone.
 constexpr int kLineMost = 2048, kLineWarps = 4;
