@@ -18,7 +18,7 @@
 // are the same bits), so the slots that atomics hand out do not show. Where a line
 // has more than kLineMost crossings the buckets go to radix sorts by x and then by
 // key; so do, without buckets, more lines than vertices (where the lines' counts
-// cost more than the crossings) and few lines for many vertices (kLineVerts).
+// cost more than the crossings).
 #include <math.h>
 #include <string.h>
 
@@ -69,6 +69,7 @@ struct HatchConst {
     const float* ys;   // the lines' y (k_line_table)
     float y0f, inv_sp;
     int32_t n_lines;
+    int32_t log_copies;   // log2 of a line's counters (count_copies)
     int64_t n_verts;
 };
 
@@ -132,18 +133,21 @@ __device__ __forceinline__ float float_of(uint32_t k) {
     return __uint_as_float((k & 0x80000000u) ? k & 0x7fffffffu : ~k);
 }
 
-// Every crossing of every edge, by whole warps: f(key, m, a, b, peers), peers = the
-// lanes that are at a crossing of the same line now. Contours list their loops row
+// Every crossing of every edge, by whole warps: f(slot, m, a, b, peers), slot = the line's
+// key << log_copies | the warp's copy of its counter, peers = the lanes that are at a
+// crossing of the same line now. Contours list their loops row
 // by row, so the lanes of a warp meet the same few lines: an atomic for each group
 // of them instead of one per crossing takes 0.13 ms instead of 1.25 for the counts
 // of 3000 x 1000 squares (12 million crossings on 2,000 lines), which one address
 // after another had held up. Edges of more than kWideEdge lines are taken by all
-// lanes together, those of more than kLongEdge are only handed to long_edge(v, lines):
+// lanes together where that is the shorter way, those of more than kLongEdge are only handed to long_edge(v, lines):
 // for the whole grid (each_long_crossing). kPerLane edges per lane at a time: the infill of
 // 389 million vertices, three in four of whose edges cross no line, takes 11.4 ms with
-// 1, 10.8 with 2 (10.9 with an atomic per crossing), 12.1 with 3 (registers).
-constexpr int kWideEdge = 32, kLongEdge = 1024, kPerLane = 2;
-template <class F, class G>
+// 1, 10.4 with 2 (11.0 where k_line_emit has 48 registers, not 40), 12.1 with 3, 11.0 with
+// an atomic per crossing; 2 from 2^22 vertices on, where the lanes have more edges than
+// one.
+constexpr int kWideEdge = 32, kLongEdge = 1024;
+template <int kPerLane, class F, class G>
 __device__ __forceinline__ void each_crossing(const float2* __restrict__ xy,
                                               const int64_t* __restrict__ loop_off,
                                               const uint32_t* __restrict__ loop_of,
@@ -153,6 +157,9 @@ __device__ __forceinline__ void each_crossing(const float2* __restrict__ xy,
     const int64_t stride = (int64_t)gridDim.x * blockDim.x * kPerLane;
     for (int64_t v0 = ((int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31u)) * kPerLane;
          v0 < c.n_verts; v0 += stride) {
+        bool any = false;
+        const uint32_t copy =
+            (uint32_t)((uint64_t)v0 / (32 * kPerLane)) & ((1u << c.log_copies) - 1u);
         // kPerLane edges per lane: their chains of loads run side by side
         float2 ea[kPerLane], eb[kPerLane];
         int em[kPerLane], en[kPerLane];
@@ -188,15 +195,27 @@ __device__ __forceinline__ void each_crossing(const float2* __restrict__ xy,
             eb[u] = b;
             em[u] = m;
             en[u] = n;
+            any |= n > 0;
         }
+        if (!__any_sync(0xffffffffu, any)) continue;
 #pragma unroll
         for (int u = 0; u < kPerLane; ++u) {
             const float2 a = ea[u], b = eb[u];
             const int m = em[u];
             const uint32_t base = ebase[u];
             int n = en[u];
-            const int most = __reduce_max_sync(0xffffffffu, n);
-            uint32_t wide = most > kWideEdge ? __ballot_sync(0xffffffffu, n > kWideEdge) : 0u;
+            int most = __reduce_max_sync(0xffffffffu, n);
+            uint32_t wide = 0u;
+            if (most > kWideEdge) {
+                // steps by all lanes together against steps of a lane per edge (which share
+                // atomics with their neighbours)
+                const int together =
+                    __reduce_add_sync(0xffffffffu, n > kWideEdge ? (n + 31) / 32 : 0);
+                if (2 * together < most) {
+                    wide = __ballot_sync(0xffffffffu, n > kWideEdge);
+                    most = kWideEdge;
+                }
+            }
             for (; wide; wide &= wide - 1u) {
                 const int src = __ffs(wide) - 1;
                 const float2 p = make_float2(__shfl_sync(0xffffffffu, a.x, src),
@@ -207,15 +226,16 @@ __device__ __forceinline__ void each_crossing(const float2* __restrict__ xy,
                 const int from = __shfl_sync(0xffffffffu, m, src);
                 const int pn = __shfl_sync(0xffffffffu, n, src);
                 for (int k = lane; k < pn; k += 32)
-                    f(pb + (uint32_t)(from + k), from + k, p, q, 1u << lane);
+                    f((pb + (uint32_t)(from + k)) << c.log_copies | copy, from + k, p, q,
+                      1u << lane);
                 if (lane == src) n = 0;
                 __syncwarp();
             }
-            for (int k = 0; k < min(most, kWideEdge); ++k) {
+            for (int k = 0; k < most; ++k) {
                 const uint32_t act = __ballot_sync(0xffffffffu, k < n);
                 if (k < n) {
-                    const uint32_t key = base + (uint32_t)(m + k);
-                    f(key, m + k, a, b, __match_any_sync(act, key));
+                    const uint32_t slot = (base + (uint32_t)(m + k)) << c.log_copies | copy;
+                    f(slot, m + k, a, b, __match_any_sync(act, slot));
                 }
             }
         }
@@ -248,22 +268,24 @@ __device__ __forceinline__ void each_long_crossing(const float2* __restrict__ xy
         const int64_t from = m0 + (int64_t)e.y * kLongEdge;
         const int64_t to = min((int64_t)m1, from + kLongEdge);
         for (int64_t m = from + threadIdx.x; m < to; m += blockDim.x)
-            f(base + (uint32_t)m, (int)m, a, b, 1u << (threadIdx.x & 31));
+            f((base + (uint32_t)m) << c.log_copies | (i & ((1u << c.log_copies) - 1u)), (int)m, a,
+              b, 1u << (threadIdx.x & 31));
     }
 }
 
 // Crossings per line; the pieces of long edges are listed (n_list[0], room for `cap` of
 // them: more have more crossings together than the call takes, n_list[1]).
+template <int U>
 __global__ void k_line_count(const float2* __restrict__ xy, const int64_t* __restrict__ loop_off,
                              const uint32_t* __restrict__ loop_of,
                              const uint32_t* __restrict__ layer_of, HatchConst c,
                              uint32_t* __restrict__ hist, uint2* __restrict__ list,
                              uint32_t cap, uint32_t* __restrict__ n_list) {
     const uint32_t lane = threadIdx.x & 31;
-    each_crossing(
+    each_crossing<U>(
         xy, loop_off, loop_of, layer_of, c,
-        [&](uint32_t key, int, float2, float2, uint32_t peers) {
-            if (lane == __ffs(peers) - 1u) atomicAdd(hist + key, (uint32_t)__popc(peers));
+        [&](uint32_t slot, int, float2, float2, uint32_t peers) {
+            if (lane == __ffs(peers) - 1u) atomicAdd(hist + slot, (uint32_t)__popc(peers));
         },
         [&](int64_t v, int lines) {
             const uint32_t n = ((uint32_t)lines + kLongEdge - 1u) / kLongEdge;
@@ -280,17 +302,20 @@ __global__ void k_line_count_long(const float2* __restrict__ xy,
                                   uint32_t* __restrict__ hist, const uint2* __restrict__ list,
                                   uint32_t cap, const uint32_t* __restrict__ n_list) {
     each_long_crossing(xy, loop_off, loop_of, layer_of, c, list, min(*n_list, cap),
-                       [&](uint32_t key, int, float2, float2, uint32_t) { atomicAdd(hist + key, 1u); });
+                       [&](uint32_t slot, int, float2, float2, uint32_t) { atomicAdd(hist + slot, 1u); });
 }
 
 // most[0] = the longest line's crossings; a line with an odd count is reported.
-__global__ void k_line_most(const uint32_t* __restrict__ hist, int64_t n_keys,
+__global__ void k_line_most(const uint32_t* __restrict__ hist, int64_t n_keys, int log_copies,
                             uint32_t* __restrict__ status, uint32_t* __restrict__ most) {
     uint32_t m = 0, odd = 0;
     for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n_keys;
          k += (int64_t)gridDim.x * blockDim.x) {
-        m = max(m, hist[k]);
-        odd |= hist[k] & 1u;
+        uint32_t n = 0;
+#pragma unroll 8
+        for (int u = 0; u < 1 << log_copies; ++u) n += hist[(k << log_copies) + u];
+        m = max(m, n);
+        odd |= n & 1u;
     }
     m = __reduce_max_sync(0xffffffffu, m);
     odd = __reduce_or_sync(0xffffffffu, odd);
@@ -309,28 +334,30 @@ struct LineBuckets {
     uint32_t* __restrict__ xs;
     uint32_t* __restrict__ keys;
 
-    __device__ __forceinline__ void put(const HatchConst& c, uint32_t key, int m, float2 a,
+    __device__ __forceinline__ void put(const HatchConst& c, uint32_t slot, int m, float2 a,
                                         float2 b, uint32_t peers) const {
         const uint32_t lane = threadIdx.x & 31;
         const float t = __fdiv_rn(c.ys[m] - a.y, b.y - a.y);
         const float x = fmaf(t, b.x - a.x, a.x);
         const int first = __ffs(peers) - 1;
         uint32_t left = 0;
-        if (lane == (uint32_t)first) left = atomicSub(hist + key, (uint32_t)__popc(peers));
+        if (lane == (uint32_t)first) left = atomicSub(hist + slot, (uint32_t)__popc(peers));
         left = __shfl_sync(peers, left, first);
-        const int64_t at = start[key] + left - 1 - __popc(peers & ((1u << lane) - 1u));
+        const int64_t at = start[slot] + left - 1 - __popc(peers & ((1u << lane) - 1u));
         xs[at] = keys ? __float_as_uint(x) : order_of(x);
-        if (keys) keys[at] = key;
+        if (keys) keys[at] = slot >> c.log_copies;
     }
 };
 
-__global__ void k_line_emit(const float2* __restrict__ xy, const int64_t* __restrict__ loop_off,
-                            const uint32_t* __restrict__ loop_of,
-                            const uint32_t* __restrict__ layer_of, HatchConst c, LineBuckets to) {
-    each_crossing(
+template <int U>
+__global__ void __launch_bounds__(256, 6)
+k_line_emit(const float2* __restrict__ xy, const int64_t* __restrict__ loop_off,
+            const uint32_t* __restrict__ loop_of, const uint32_t* __restrict__ layer_of,
+            HatchConst c, LineBuckets to) {
+    each_crossing<U>(
         xy, loop_off, loop_of, layer_of, c,
-        [&](uint32_t key, int m, float2 a, float2 b, uint32_t peers) {
-            to.put(c, key, m, a, b, peers);
+        [&](uint32_t slot, int m, float2 a, float2 b, uint32_t peers) {
+            to.put(c, slot, m, a, b, peers);
         },
         [](int64_t, int) {});
 }
@@ -341,8 +368,8 @@ __global__ void k_line_emit_long(const float2* __restrict__ xy,
                                  const uint32_t* __restrict__ layer_of, HatchConst c,
                                  LineBuckets to, const uint2* __restrict__ list, uint32_t n) {
     each_long_crossing(xy, loop_off, loop_of, layer_of, c, list, n,
-                       [&](uint32_t key, int m, float2 a, float2 b, uint32_t peers) {
-                           to.put(c, key, m, a, b, peers);
+                       [&](uint32_t slot, int m, float2 a, float2 b, uint32_t peers) {
+                           to.put(c, slot, m, a, b, peers);
                        });
 }
 
@@ -350,17 +377,12 @@ __global__ void k_line_emit_long(const float2* __restrict__ xy,
 // the next power of two, at most `room`) and its segments written in toolpath
 // order. 250 layers of 500 lines: 0.23 ms, bound by the latency of the loads and
 // stages (strides below 32 by shuffles instead: the same); the infill with the
-// counts (0.19 ms) and the buckets (0.34 ms) 1.03 ms a call, 1.10 with an atomic per
+// counts (0.19 ms) and the buckets (0.3 ms) 1.00 ms a call, 1.11 with an atomic per
 // crossing in both (0.23 and 0.35; 0.84 ms of kernels, where 7 passes of radix sorts
 // made 1.39). 1000 x 1000 squares x 3 layers (2,000 crossings per line): 0.90 ms, 1.68
 // with radix sorts alone; 3000 x 1000 (6,000 per line): buckets and radix sorts
 // 1.50 ms, 1.67 with radix sorts alone.
 constexpr int kLineMost = 2048, kLineWarps = 4;
-// Contours with as many vertices per line as this go straight to the radix sorts:
-// their lines are too long in all but odd cases, and so few counters are contended
-// (200,000 x 5 squares, 20 lines: 0.69 ms so, 4.4 ms with the lines counted first by an
-// atomic per crossing).
-constexpr uint64_t kLineVerts = 1 << 15;
 __global__ void __launch_bounds__(32 * kLineWarps)
 k_line_sort(const uint32_t* __restrict__ xs, const int64_t* __restrict__ start, int64_t n_keys,
             int64_t n_rec, int room, HatchConst c, float* __restrict__ out) {
@@ -370,7 +392,8 @@ k_line_sort(const uint32_t* __restrict__ xs, const int64_t* __restrict__ start, 
     const int64_t stride = (int64_t)gridDim.x * kLineWarps;
     for (int64_t k = (int64_t)blockIdx.x * kLineWarps + (threadIdx.x >> 5); k < n_keys;
          k += stride) {
-        const int64_t lo = start[k], hi = k + 1 < n_keys ? start[k + 1] : n_rec;
+        const int64_t lo = start[k << c.log_copies];
+        const int64_t hi = k + 1 < n_keys ? start[(k + 1) << c.log_copies] : n_rec;
         const int n = (int)(hi - lo);
         if (n < 2 || n > room) continue;
         int P = 2;
@@ -405,10 +428,10 @@ k_line_sort(const uint32_t* __restrict__ xs, const int64_t* __restrict__ start, 
 
 // layer_off[k] = first segment of layer k, from the lines' starts
 __global__ void k_line_offsets(const int64_t* __restrict__ start, int64_t n_rec, int n_layers,
-                               int n_lines, int64_t* __restrict__ layer_off) {
+                               int n_lines, int log_copies, int64_t* __restrict__ layer_off) {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k > n_layers) return;
-    layer_off[k] = (k == n_layers ? n_rec : start[(int64_t)k * n_lines]) / 2;
+    layer_off[k] = (k == n_layers ? n_rec : start[((int64_t)k * n_lines) << log_copies]) / 2;
 }
 
 __global__ void k_x_keys(const float* __restrict__ xs, int64_t n, uint32_t* __restrict__ k,
@@ -482,6 +505,18 @@ __global__ void k_layer_offsets(const uint32_t* __restrict__ seg_key, int64_t n_
     layer_off[k] = k == n_layers ? n_seg : lo;
 }
 
+// log2 of the counters of a line: few lines of many vertices lie in a few sectors of
+// L2, where atomics take turns whatever their address, so each line gets up to 64
+// counters (its bucket is one part per counter) while there are no more than 2^14 in
+// all and 128 vertices for each. 100,000 squares, 50 lines: 1.04 ms, 2.4 with one counter, 1.14
+// with radix sorts alone; 200,000 x 5 squares, 20 lines: 0.77, 1.12 and 0.89.
+int count_copies(int64_t n_keys, int64_t n_verts) {
+    const int64_t most = n_verts / 128 < 1 << 14 ? n_verts / 128 : 1 << 14;
+    int log = 0;
+    while (log < 6 && n_keys << (log + 1) <= most) ++log;
+    return log;
+}
+
 int bits_for(uint64_t n) {
     int b = 1;
     while (b < 32 && ((uint64_t)1 << b) < n) ++b;
@@ -517,7 +552,7 @@ csl_status csl_hatch_layers(const csl_contours* ct, double y0, double spacing, i
                                                                          ys_d.as<float>());
             CSL_LAUNCH_CHECK("hatch lines");
         }
-        HatchConst c{ys_d.as<float>(), (float)y0, (float)(1.0 / spacing), n_lines, n_verts};
+        HatchConst c{ys_d.as<float>(), (float)y0, (float)(1.0 / spacing), n_lines, 0, n_verts};
         const float2* xy = reinterpret_cast<const float2*>(ct->xy);
 
         int64_t n_rec = 0;
@@ -543,16 +578,21 @@ csl_status csl_hatch_layers(const csl_contours* ct, double y0, double spacing, i
             CSL_LAUNCH_CHECK("hatch layer of loop");
             // the first loops may precede the first layer start only when layer 0
             // has loops; layer_loop_off[0] is 0, so the counts are the layers
-            if (n_keys <= (uint64_t)n_verts && (uint64_t)n_verts / n_keys < kLineVerts) {
-                DevBuf hist((size_t)n_keys * 4, s);
-                CSL_CUDA(cudaMemsetAsync(hist.get(), 0, (size_t)n_keys * 4, s));
+            if (n_keys <= (uint64_t)n_verts) {
+                c.log_copies = count_copies((int64_t)n_keys, n_verts);
+                const int64_t n_slots = (int64_t)n_keys << c.log_copies;
+                DevBuf hist((size_t)n_slots * 4, s);
+                CSL_CUDA(cudaMemsetAsync(hist.get(), 0, (size_t)n_slots * 4, s));
                 // pieces of long edges: at least half of each is lines that it crosses, so
                 // this many hold all the crossings that a call may have
                 const int64_t pieces = ceil_div(n_lines, kLongEdge);
                 const uint32_t long_cap = n_lines <= kLongEdge ? 0u
                     : (uint32_t)std::min<int64_t>(n_verts * pieces, (2ll << 32) / kLongEdge);
                 DevBuf long_edges((size_t)std::max(long_cap, 1u) * 8, s);
-                k_line_count<<<grid_for(n_verts, 256), 256, 0, s>>>(
+                const bool two = n_verts >= (1 << 22);
+                auto line_count = two ? k_line_count<2> : k_line_count<1>;
+                auto line_emit = two ? k_line_emit<2> : k_line_emit<1>;
+                line_count<<<grid_for(n_verts, 256), 256, 0, s>>>(
                     xy, ct->loop_vert_off, loop_of.as<uint32_t>(), layer_of.as<uint32_t>(), c,
                     hist.as<uint32_t>(), long_edges.as<uint2>(), long_cap,
                     small.as<uint32_t>() + 4);
@@ -565,12 +605,12 @@ csl_status csl_hatch_layers(const csl_contours* ct, double y0, double spacing, i
                     CSL_LAUNCH_CHECK("hatch line counts of long edges");
                 }
                 k_line_most<<<grid_for((int64_t)n_keys, 256), 256, 0, s>>>(
-                    hist.as<uint32_t>(), (int64_t)n_keys, small.as<uint32_t>() + 2,
+                    hist.as<uint32_t>(), (int64_t)n_keys, c.log_copies, small.as<uint32_t>() + 2,
                     small.as<uint32_t>() + 3);
                 CSL_LAUNCH_CHECK("hatch longest line");
-                line_start.alloc((size_t)n_keys * 8, s);
-                exclusive_scan_u32_to_i64(hist.as<uint32_t>(), line_start.as<int64_t>(),
-                                          (int64_t)n_keys, small.as<int64_t>(), s);
+                line_start.alloc((size_t)n_slots * 8, s);
+                exclusive_scan_u32_to_i64(hist.as<uint32_t>(), line_start.as<int64_t>(), n_slots,
+                                          small.as<int64_t>(), s);
                 uint32_t h[6];
                 read_to_host(h, small.get(), sizeof h, s);
                 n_rec = (int64_t)(((uint64_t)h[1] << 32) | h[0]);
@@ -584,7 +624,7 @@ csl_status csl_hatch_layers(const csl_contours* ct, double y0, double spacing, i
                     if (!by_line) key.alloc((size_t)n_rec * 4, s);
                     const LineBuckets to{line_start.as<int64_t>(), hist.as<uint32_t>(),
                                          xs.as<uint32_t>(), by_line ? nullptr : key.as<uint32_t>()};
-                    k_line_emit<<<grid_for(n_verts, 256), 256, 0, s>>>(
+                    line_emit<<<grid_for(n_verts, 256), 256, 0, s>>>(
                         xy, ct->loop_vert_off, loop_of.as<uint32_t>(), layer_of.as<uint32_t>(), c,
                         to);
                     CSL_LAUNCH_CHECK("hatch line crossings");
@@ -643,7 +683,8 @@ csl_status csl_hatch_layers(const csl_contours* ct, double y0, double spacing, i
                     c, segs.as<float>());
                 CSL_LAUNCH_CHECK("hatch line sort");
                 k_line_offsets<<<(unsigned)ceil_div(n_layers + 1, 128), 128, 0, s>>>(
-                    line_start.as<int64_t>(), n_rec, (int)n_layers, n_lines, lay.as<int64_t>());
+                    line_start.as<int64_t>(), n_rec, (int)n_layers, n_lines, c.log_copies,
+                    lay.as<int64_t>());
                 CSL_LAUNCH_CHECK("hatch layer offsets");
             } else if (n_seg > 0) {
                 // sort by x, then (stably) by line key

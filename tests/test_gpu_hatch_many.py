@@ -1,6 +1,6 @@
 """Infill of rows of bars whose neighbours cross the same lines: short and long lines, sides
-of more lines than a warp has lanes, and so many vertices per line that the lines are not
-counted. Vertical sides, so that every crossing's x is a side's x exactly."""
+of more lines than a warp has lanes, and so many vertices per line that each line has several
+counters. Vertical sides, so that every crossing's x is a side's x exactly."""
 import numpy as np
 import pytest
 
@@ -20,6 +20,8 @@ def _rows(per_row, rows, height):
     ([np.concatenate([_rows(300, 20, 0.6), _rows(5, 1, 33.0) - [7.5, 0, 0, 0]])] * 2, 500, 0.07),
     ([_rows(1100, 1, 30.0)], 90, 0.31),               # long lines, sides of 97 lines
     ([_rows(9000, 1, 0.6)], 1, 0.3),                  # 36,000 vertices for one line
+    ([_rows(500, 4, 0.6)] * 3, 13, 0.045),            # sides of 13 lines, 16 counters per line
+    ([_rows(400, 1, 2.0)] * 2, 48, 0.04),             # sides of 48 lines by their own lanes
     # sides of 1024, 1025, 2049 and 3,300 lines beside short ones; in lines too long for a warp
     ([np.concatenate([_rows(40, 60, 0.6), [[-2, 0, 0.5, 30.705], [-4, 0, 0.5, 30.735],
                                            [-6, 3, 0.5, 61.455], [-8, 0, 0.5, 99.0]]])] * 2, 3400, 0.03),
