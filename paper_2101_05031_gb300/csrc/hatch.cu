@@ -133,19 +133,19 @@ __device__ __forceinline__ float float_of(uint32_t k) {
     return __uint_as_float((k & 0x80000000u) ? k & 0x7fffffffu : ~k);
 }
 
-// Every crossing of every edge, by whole warps: f(slot, m, a, b, peers), slot = the line's
-// key << log_copies | the warp's copy of its counter, peers = the lanes that are at a
-// crossing of the same line now. Contours list their loops row
-// by row, so the lanes of a warp meet the same few lines: an atomic for each group
-// of them instead of one per crossing takes 0.13 ms instead of 1.25 for the counts
-// of 3000 x 1000 squares (12 million crossings on 2,000 lines), which one address
-// after another had held up. Edges of more than kWideEdge lines are taken by all
-// lanes together where that is the shorter way, those of more than kLongEdge are only handed to long_edge(v, lines):
-// for the whole grid (each_long_crossing). kPerLane edges per lane at a time: the infill of
+// Every crossing of every edge, by whole warps: f(slot, m, a, b, peers), slot = the
+// line's key << log_copies | the warp's copy of its counter, peers = the lanes that are
+// at a crossing of the same line now. Contours list their loops row by row, so the
+// lanes of a warp meet the same few lines: an atomic for each group of them instead of
+// one per crossing takes 0.13 ms instead of 1.25 for the counts of 3000 x 1000 squares
+// (12 million crossings on 2,000 lines), where atomics on one address took turns. Edges
+// of more than kWideEdge lines are taken by all lanes together where that is the
+// shorter way, those of more than kLongEdge are only handed to long_edge(v, lines): for
+// the whole grid (each_long_crossing). kPerLane edges per lane at a time: the infill of
 // 389 million vertices, three in four of whose edges cross no line, takes 11.4 ms with
-// 1, 10.4 with 2 (11.0 where k_line_emit has 48 registers, not 40), 12.1 with 3, 11.0 with
-// an atomic per crossing; 2 from 2^22 vertices on, where the lanes have more edges than
-// one.
+// 1, 10.4 with 2 (11.0 where k_line_emit has 48 registers, not 40), 12.1 with 3, 11.0
+// with an atomic per crossing; 2 from 2^22 vertices on, where the lanes have more edges
+// than one.
 constexpr int kWideEdge = 32, kLongEdge = 1024;
 template <int kPerLane, class F, class G>
 __device__ __forceinline__ void each_crossing(const float2* __restrict__ xy,
